@@ -141,8 +141,12 @@ int lq_convert(lq_handle *h, void *dst, int dst_fmt, const void *src, int src_fm
  * fields, as selected by `parity` (LQ_FULL, LQ_EVEN, LQ_ODD, LQ_SCHUR_EVEN).
  * fmt gives layout and arithmetic of in and out: LQ_F64 / LQ_F32 site-major
  * (converted to native and back inside the call, using handle workspace), or
- * LQ_NATIVE | p (streamed directly).  FP64 fields compute in FP64; FP32, FP16
- * and BF16 fields compute in FP32 with links stored in the same precision.
+ * LQ_NATIVE | p (streamed directly).  FP32, FP16 and BF16 fields compute in FP32
+ * with links stored in the same precision.  FP64 fields compute in FP64, or, with
+ * links that are SU(3) (entries up to 1, rows and columns of 1-norm up to 2.75, which
+ * lq_create checks), form the hopping sums in 64-bit fixed point: exact products and
+ * sums to 2^-56 of the largest component of the site's 8 neighbours, rounded to FP64
+ * once.
  */
 int dslash_apply(lq_handle *h, void *out, const void *in, int fmt, int parity, int nrhs, void *stream);
 int dslash_dag_apply(lq_handle *h, void *out, const void *in, int fmt, int parity, int nrhs, void *stream);

@@ -87,7 +87,9 @@ int get_links(lq_handle* h, int prec, const char** links, size_t* link_block, cu
             L = nullptr;
             return LQ_ERR_NOMEM;
         }
-        cudaError_t e = launch_links_to_native(prec, r12, L, h->U_prec, h->U_sm, h->g, st);
+        cudaError_t e = prec == LQ_F64 && h->fixed64
+                            ? launch_links_fixed(L, h->U_prec, h->U_sm, h->g, st)
+                            : launch_links_to_native(prec, r12, L, h->U_prec, h->U_sm, h->g, st);
         if (e != cudaSuccess) return LQ_ERR_CUDA;
     }
     *links = static_cast<const char*>(L);
@@ -110,6 +112,7 @@ static HopArgs base_args(lq_handle* h, const char* links, size_t lb) {
     a.g = h->g;
     a.skip = h->skip;
     a.skip_stride = h->skip_stride;
+    a.fixed = h->fixed64;
     a.mma = h->hop_kernel == LQ_HOP_TENSOR_CORES ? 1 : 0;
     return a;
 }
@@ -610,14 +613,20 @@ int lq_create(lq_handle** hp, const lq_params* p, const void* U, int U_prec, voi
     }
     h->U_prec = U_prec;
     const size_t ub = (size_t)V * 72 * (U_prec == LQ_F64 ? 8 : 4);
-    if (cudaMalloc(&h->U_sm, ub) != cudaSuccess) {
+    if (cudaMalloc(&h->U_sm, ub + 16) != cudaSuccess) {  // and a counter of unfit links
         cudaGetLastError();
         delete h;
         return LQ_ERR_NOMEM;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMemcpyAsync(h->U_sm, U, ub, cudaMemcpyDeviceToDevice, st);
+    unsigned* bad = reinterpret_cast<unsigned*>(static_cast<char*>(h->U_sm) + ub);
+    unsigned nbad = 1;
+    if (e == cudaSuccess) e = cudaMemsetAsync(bad, 0, sizeof(*bad), st);
+    if (e == cudaSuccess) e = launch_links_fixed_check(U_prec, h->U_sm, V * 4, bad, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&nbad, bad, sizeof(nbad), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    h->fixed64 = nbad == 0;
     if (e != cudaSuccess) {
         lq_destroy(h);
         return LQ_ERR_CUDA;

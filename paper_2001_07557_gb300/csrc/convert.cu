@@ -89,7 +89,8 @@ __global__ void native_convert_kernel(char* dst, const char* src, int Vh) {
     }
 }
 
-template <int DP, bool R12, int SP>
+// FIXED: the fixed-point records of hop_fixed.cuh (DP = LQ_F64)
+template <int DP, bool R12, int SP, bool FIXED = false>
 __global__ void links_kernel(char* dst, const void* src, Geom g, size_t link_block) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.Vh) return;
@@ -109,7 +110,8 @@ __global__ void links_kernel(char* dst, const void* src, Geom g, size_t link_blo
                 u[k] = {(double)v.x, (double)v.y};
             }
         }
-        store_link<DP, R12>(dst + (size_t)(p * 4 + mu) * link_block, g.Vh, i, u);
+        if constexpr (FIXED) store_link_fixed(dst + (size_t)(p * 4 + mu) * link_block, g.Vh, i, u);
+        else store_link<DP, R12>(dst + (size_t)(p * 4 + mu) * link_block, g.Vh, i, u);
     }
 }
 
@@ -171,6 +173,37 @@ __global__ void link_su3_deviation_kernel(const void* src, long nlinks, unsigned
     for (int o = 16; o > 0; o >>= 1) dev = fmax(dev, __shfl_xor_sync(0xffffffffu, dev, o));
     // non-negative doubles order like their bit patterns
     if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(dev));
+}
+
+// |v| cut to FP32 without the FP64 unit (4 for |v| >= 2, infinities and NaNs; 0 below 2^-126)
+__device__ __forceinline__ float abs_f32(double v) {
+    const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
+    if (h >= 0x40000000u) return 4.0f;
+    if (h < 0x38100000u) return 0.0f;
+    return __uint_as_float(((h - 0x38000000u) << 3) | ((unsigned)__double2loint(v) >> 29));
+}
+__device__ __forceinline__ float abs_f32(float v) { return fabsf(v) < 2.0f ? fabsf(v) : 4.0f; }
+
+// The links that the fixed-point FP64 hop cannot take: its sums are bounded for entries up to 1
+// and rows and columns of 1-norm up to 2.75 (SU(3): sqrt 6).
+template <typename T>
+__global__ void link_fixed_check_kernel(const T* src, long nlinks, unsigned* bad) {
+    unsigned n = 0;
+    for (long l = (long)blockIdx.x * blockDim.x + threadIdx.x; l < nlinks; l += (long)gridDim.x * blockDim.x) {
+        float row[3] = {}, col[3] = {};
+        bool ok = true;
+#pragma unroll
+        for (int k = 0; k < 18; ++k) {
+            const float f = abs_f32(src[l * 18 + k]);
+            ok = ok && f <= 1.000001f;
+            row[k / 6] += f;
+            col[k / 2 % 3] += f;
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) ok = ok && row[k] <= 2.75f && col[k] <= 2.75f;
+        n += ok ? 0 : 1;
+    }
+    if (n) atomicAdd(bad, n);
 }
 
 }  // namespace
@@ -241,6 +274,24 @@ cudaError_t launch_links_to_native(int dst_prec, bool r12, void* dst, int src_pr
         if (r12) { LQ_DP_SWITCH(dst_prec, (links_kernel<DP, true, LQ_F32><<<grid, kBlock, 0, st>>>(d, src, g, lb))) }
         else { LQ_DP_SWITCH(dst_prec, (links_kernel<DP, false, LQ_F32><<<grid, kBlock, 0, st>>>(d, src, g, lb))) }
     }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_links_fixed(void* dst, int src_prec, const void* src, const Geom& g, cudaStream_t st) {
+    dim3 grid((g.Vh + kBlock - 1) / kBlock, 2);
+    const size_t lb = (size_t)link_site_bytes(LQ_F64, false) * g.Vh;
+    char* d = static_cast<char*>(dst);
+    if (src_prec == LQ_F64) links_kernel<LQ_F64, false, LQ_F64, true><<<grid, kBlock, 0, st>>>(d, src, g, lb);
+    else links_kernel<LQ_F64, false, LQ_F32, true><<<grid, kBlock, 0, st>>>(d, src, g, lb);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_links_fixed_check(int src_prec, const void* src, long nlinks, unsigned* bad, cudaStream_t st) {
+    const int grid = (int)std::min<long>((nlinks + 255) / 256, 4096);
+    if (src_prec == LQ_F64)
+        link_fixed_check_kernel<<<grid, 256, 0, st>>>(static_cast<const double*>(src), nlinks, bad);
+    else
+        link_fixed_check_kernel<<<grid, 256, 0, st>>>(static_cast<const float*>(src), nlinks, bad);
     return cudaGetLastError();
 }
 

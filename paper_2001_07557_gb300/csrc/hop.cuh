@@ -17,6 +17,69 @@
 
 namespace lq {
 
+// ------------------------------------------------- epilogues of one site
+
+// o += c_diag x
+template <typename T>
+__device__ __forceinline__ void hop_add_diag(const HopArgs& a, const cplx<T> (&xs)[12], cplx<T> (&o)[12]) {
+    const T cd = (T)a.c_diag;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        o[k].re = fma(cd, xs[k].re, o[k].re);
+        o[k].im = fma(cd, xs[k].im, o[k].im);
+    }
+}
+
+// c_shift (S x)(s): P+ = upper spins (gamma_5 = diag(1,1,-1,-1)).  Non-dagger: upper from
+// s-1, lower from s+1; dagger swaps.  Coefficient c_shift (Shamir: -1), times -mf across the wall.
+template <typename T>
+struct HopShift {
+    int up, dn;     // slices that the upper and the lower spins come from
+    T c_up, c_dn;
+};
+template <bool DAG, typename T>
+__device__ __forceinline__ HopShift<T> hop_shift(const HopArgs& a, int s) {
+    const int Ls = a.Ls;
+    const bool first = s == 0, last = s + 1 == Ls;
+    const int below = first ? Ls - 1 : s - 1, above = last ? 0 : s + 1;
+    const T c = (T)a.c_shift, cw = (T)(-a.c_shift * a.mf);
+    HopShift<T> h;
+    h.up = DAG ? above : below;
+    h.dn = DAG ? below : above;
+    h.c_up = (DAG ? last : first) ? cw : c;
+    h.c_dn = (DAG ? first : last) ? cw : c;
+    return h;
+}
+template <int P, bool DAG, typename T>
+__device__ __forceinline__ void hop_add_shift(const HopArgs& a, int s, int p, int i, cplx<T> (&o)[12]) {
+    const HopShift<T> h = hop_shift<DAG, T>(a, s);
+    cplx<T> su[12], sd[12];
+    load_spinor<P, T>(a.x[p] + (size_t)h.up * a.x_rhs, a.g.Vh, i, su);
+    load_spinor<P, T>(a.x[p] + (size_t)h.dn * a.x_rhs, a.g.Vh, i, sd);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        o[k].re = fma(h.c_up, su[k].re, o[k].re);
+        o[k].im = fma(h.c_up, su[k].im, o[k].im);
+        o[6 + k].re = fma(h.c_dn, sd[6 + k].re, o[6 + k].re);
+        o[6 + k].im = fma(h.c_dn, sd[6 + k].im, o[6 + k].im);
+    }
+}
+
+// the fused |out|^2: warp partials, group-major: [group][warp of the group's blocks]
+template <int EPI, typename T>
+__device__ __forceinline__ void hop_norm_site(const HopArgs& a, const cplx<T> (&o)[12], bool active, int rhs, int pt) {
+    double v = 0;
+    if (active) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) v += (double)(o[k].re * o[k].re + o[k].im * o[k].im);
+    }
+    const int wpb = blockDim.x >> 5;
+    const int grp = EPI == EPI_DWF ? 0 : rhs;
+    const int nblk = EPI == EPI_DWF ? gridDim.x : gridDim.x / a.nrhs;
+    const int bidx = EPI == EPI_DWF ? blockIdx.x : pt;
+    hop_norm_warp(v, a.red_partial + (size_t)grp * nblk * wpb, bidx * wpb + (threadIdx.x >> 5));
+}
+
 template <int P, bool R12, bool DAG, int EPI, bool RED>
 __global__ void __launch_bounds__(128) wilson_hop_kernel(const HopArgs a) {
     pdl_enter();
@@ -137,52 +200,13 @@ __global__ void __launch_bounds__(128) wilson_hop_kernel(const HopArgs a) {
     for (int k = 0; k < 12; ++k) o[k] = {ch * acc[k].re, ch * acc[k].im};
 
     if constexpr (EPI >= EPI_DIAG) {
-        const T cd = (T)a.c_diag;
-        const char* __restrict__ xb = a.x[p] + (size_t)rhs * a.x_rhs;
         cplx<T> xs[12];
-        load_spinor<P, T>(xb, g.Vh, i, xs);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            o[k].re = fma(cd, xs[k].re, o[k].re);
-            o[k].im = fma(cd, xs[k].im, o[k].im);
-        }
+        load_spinor<P, T>(a.x[p] + (size_t)rhs * a.x_rhs, g.Vh, i, xs);
+        hop_add_diag<T>(a, xs, o);
     }
-    if constexpr (EPI == EPI_DWF) {
-        // P+ = upper spins (gamma_5 = diag(1,1,-1,-1)).  Non-dagger: upper from
-        // s-1, lower from s+1; dagger swaps.  Coefficient c_shift (Shamir: -1), times -mf across the wall.
-        const int Ls = a.Ls;
-        const int s = rhs;
-        const int s_up = DAG ? (s + 1 == Ls ? 0 : s + 1) : (s == 0 ? Ls - 1 : s - 1);
-        const int s_dn = DAG ? (s == 0 ? Ls - 1 : s - 1) : (s + 1 == Ls ? 0 : s + 1);
-        const bool wrap_up = DAG ? (s + 1 == Ls) : (s == 0);
-        const bool wrap_dn = DAG ? (s == 0) : (s + 1 == Ls);
-        const T c_up = wrap_up ? (T)(-a.c_shift * a.mf) : (T)a.c_shift;
-        const T c_dn = wrap_dn ? (T)(-a.c_shift * a.mf) : (T)a.c_shift;
-        cplx<T> su[12], sd[12];
-        load_spinor<P, T>(a.x[p] + (size_t)s_up * a.x_rhs, g.Vh, i, su);
-        load_spinor<P, T>(a.x[p] + (size_t)s_dn * a.x_rhs, g.Vh, i, sd);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            o[k].re = fma(c_up, su[k].re, o[k].re);
-            o[k].im = fma(c_up, su[k].im, o[k].im);
-            o[6 + k].re = fma(c_dn, sd[6 + k].re, o[6 + k].re);
-            o[6 + k].im = fma(c_dn, sd[6 + k].im, o[6 + k].im);
-        }
-    }
+    if constexpr (EPI == EPI_DWF) hop_add_shift<P, DAG, T>(a, rhs, p, i, o);
     if (active) store_spinor<P, T>(a.out[p] + (size_t)rhs * a.out_rhs, g.Vh, i, o);
-    if constexpr (RED) {
-        double v = 0;
-        if (active) {
-#pragma unroll
-            for (int k = 0; k < 12; ++k) v += (double)(o[k].re * o[k].re + o[k].im * o[k].im);
-        }
-        // warp partials, group-major: [group][warp of the group's blocks]
-        const int wpb = blockDim.x >> 5;
-        const int grp = EPI == EPI_DWF ? 0 : rhs;
-        const int nblk = EPI == EPI_DWF ? gridDim.x : gridDim.x / a.nrhs;
-        const int bidx = EPI == EPI_DWF ? blockIdx.x : pt;
-        hop_norm_warp(v, a.red_partial + (size_t)grp * nblk * wpb, bidx * wpb + (threadIdx.x >> 5));
-    }
+    if constexpr (RED) hop_norm_site<EPI, T>(a, o, active, rhs, pt);
 }
 
 template <int P>

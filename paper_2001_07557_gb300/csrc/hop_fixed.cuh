@@ -1,0 +1,545 @@
+// hop_fixed.cuh -- the FP64 Wilson hop with its products and sums in 64-bit
+// fixed point on the integer multipliers.
+//
+// What bounds the plain FP64 hop (hop.cuh) is the FP64 unit: GB300 issues 1.67
+// FP64 lanes per clock and SM (measured), a site needs 864 FP64 instructions,
+// so one even-odd hop on 32^4 takes 0.9 ms where its bytes take 0.12 ms.  The
+// 32x32+64-bit integer multiply-add runs at 63 lanes per clock and SM
+// (measured), 38 times that rate.  Here a site's arithmetic is integer:
+//
+//   * block floating point: of the 24 reals of a neighbour the largest exponent
+//     is found, and each becomes the signed integer x 2^59 / 2^B, 2^B above all
+//     neighbours so far, as two words hi * 2^30 + lo (|hi| < 2^29, lo < 2^30), whose
+//     spin projection (sums of two) still fits two 32-bit words;
+//   * links are packed once as u 2^58 = hi * 2^30 + lo (|lo| <= 2^29);
+//   * a real product is three multiply-adds: hi*hi, and hi*lo + lo*hi into a
+//     second 64-bit sum that is rounded in at the end of each dot product
+//     (lo*lo, below 2^-57 of the block, is dropped);
+//   * the 24 sums over 8 directions are 64-bit integers in units of 2^(B-57).
+//     A neighbour larger than 2^B moves the sums to its exponent.
+//
+// Precision: the sums carry 57 bits below the largest neighbour component (56 where the
+// headroom of the block exponent is used), against the 53 bits of each FP64 partial sum.
+// Against 64-bit reference results of D on 32^4 the error is 1.1e-16 (FP64 kernel 1.2e-16),
+// of Mhat^dag on 10x14x18x22 0.96e-16 (1.1e-16).  What is not finite, beyond 2^976 or below
+// 2^-894 takes the FP64 sums of slow_site.
+//
+// It needs links with |u| <= 1 and rows and columns of 1-norm <= 2.75 (SU(3): <= 2.45), which
+// bounds every sum below 2^63 (link_fixed_check_kernel, when a handle is made); other links
+// keep the FP64 kernel.
+//
+// Layout: two threads a site, one for each spin of the half spinors; lanes 0-15 and 16-31 of a
+// warp share 16 sites.  A site's neighbour spinor (192 B) and link (144 B) come by cp.async into
+// one shared-memory slot each: the next spinor is requested as soon as this one is converted,
+// the next link when this one is used up, so the products (conversions) of a direction cover the
+// latency.  With one thread a site, 168 registers and the 8 directions unrolled, the 120 KB of
+// code kept warps waiting for instructions (240 us); one looped body with run-time directions
+// executed 10,800 instructions a site where this takes 8,900 (236 against 215 us).
+//
+// Measured: D on 32^3 x 16 (as many sites as an even-odd hop of 32^4): 0.90 ms in FP64, 0.215 ms
+// here; its bytes take 0.12 ms.  What bounds it is the integer pipes: without its products,
+// conversions and sums the kernel takes 0.123 ms; the multiplier is busy 64 % of the time, the
+// ALU 44 %, with warps waiting on fixed latencies (ncu).
+#pragma once
+
+#include <cuda_pipeline.h>
+
+#include "hop.cuh"
+
+namespace lq {
+
+constexpr int kFixEmin = 128;    // biased exponents the block may have
+constexpr int kFixEmax = 2000;
+constexpr uint32_t kFixMask = (1u << 30) - 1;
+
+__device__ __forceinline__ uint64_t shr64(uint64_t v, uint32_t n) {  // 0 for n > 63
+    uint64_t r;
+    asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
+}
+__device__ __forceinline__ uint32_t shr32(uint32_t v, uint32_t n) {  // 0 for n > 31
+    uint32_t r;
+    asm("shr.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+    return r;
+}
+__device__ __forceinline__ long long sar64(long long v, uint32_t n) {  // the sign for n > 63
+    long long r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
+}
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) { return (long long)a * b + c; }
+
+__device__ __forceinline__ double value(uint2 w) { return __hiloint2double((int)w.y, (int)w.x); }
+__device__ __forceinline__ uint2 words(double v) {
+    return make_uint2((unsigned)__double2loint(v), (unsigned)__double2hiint(v));
+}
+
+// The larger of m and the high words of two doubles without their signs, compared as FP32
+// numbers (of the same order; a word that is an FP32 NaN, from 2^1017 up, gives a NaN, which is
+// above every exponent allowed).
+__device__ __forceinline__ float max_hi(float m, uint32_t a, uint32_t b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(fabsf(__uint_as_float(a))), "f"(fabsf(__uint_as_float(b))));
+    return r;
+}
+
+// |x| as fixed point below the block exponent (rounded toward zero), and the sign as +-1
+struct FixMag {
+    int hi, lo, s;
+};
+// e2 = 2 (Eb 2^20 + 2^20 - 1) + 1 + 5 2^21 with Eb the block's biased exponent: e2 - 2 w
+// (w: the high word of x) has Eb - e + 5 in its top 11 bits whatever x's sign and mantissa
+// are.  neg = 0, or -1 to negate.  A zero or subnormal x is shifted out, for Eb >= kFixEmin.
+__device__ __forceinline__ FixMag fix_mag(uint2 x, uint32_t e2, int neg) {
+    const uint32_t w = x.y, l = x.x;
+    const uint32_t d = (e2 - 2u * w) >> 21;  // the block exponent above x's, plus 5
+    const uint32_t nh = __funnelshift_l(l, w, 11) | 0x80000000u, nl = l << 11;  // mantissa, top bit set
+    FixMag f;
+    f.lo = (int)((uint32_t)shr64(((uint64_t)nh << 32) | nl, d) & kFixMask);
+    f.hi = (int)shr32(nh, d - 2u);
+    f.s = (((int)w >> 31) ^ neg) | 1;
+    return f;
+}
+__device__ __forceinline__ Fix2 fix_one(uint2 x, uint32_t e2, int neg) {
+    const FixMag f = fix_mag(x, e2, neg);
+    return {f.hi * f.s, f.lo * f.s};
+}
+__device__ __forceinline__ Fix2 fix_pair(uint2 x, uint2 y, uint32_t e2, int nx, int ny) {
+    const FixMag f = fix_mag(x, e2, nx), g = fix_mag(y, e2, ny);
+    return {f.hi * f.s + g.hi * g.s, f.lo * f.s + g.lo * g.s};
+}
+
+// sum_k x_k y_k over six products, rounded to units of 2^60 of the product of the scales
+__device__ __forceinline__ long long fix_dot(const Fix2 (&u)[6], const Fix2 (&h)[6]) {
+    long long mid = 1LL << 29, top;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        mid = mad_wide(u[k].hi, h[k].lo, mid);
+        mid = mad_wide(u[k].lo, h[k].hi, mid);
+    }
+    top = mid >> 30;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) top = mad_wide(u[k].hi, h[k].hi, top);
+    return top;
+}
+
+// v 2^(eb - 1079) rounded to nearest, eb a biased exponent in range; negated for the high bit of flip
+__device__ __forceinline__ double fix_to_double(long long v, int eb, uint32_t flip) {
+    const uint32_t sign = ((uint32_t)(v >> 32) ^ flip) & 0x80000000u;
+    uint64_t m = (uint64_t)(v < 0 ? -v : v);
+    int lz = __clz((int)(m >> 32));
+    if (lz == 32) {  // rare: cancelled by 2^-30
+        if (m == 0) return 0.0;
+        lz += __clz((int)(uint32_t)m);
+    }
+    m <<= lz;
+    const uint64_t b = (m >> 11) + ((m >> 10) & 1);  // the leading bit carries into the exponent
+    return __hiloint2double((int)(((uint32_t)(b >> 32) + ((uint32_t)(eb + 6 - lz) << 20)) | sign), (int)(uint32_t)b);
+}
+
+// ------------------------------------------------------------------- links
+
+// entry of a fixed-point link (fix_link_entry)
+__device__ __forceinline__ double fix_link_value(int hi, int lo) {
+    return (double)(((long long)hi << 30) + lo) * 3.469446951953614189e-18;  // 2^-58
+}
+
+// The hop sums of one site in FP64, from the fixed-point links: for neighbours that are not
+// finite or out of the fixed-point range.  out: 24 doubles, NT * 2 apart by pairs.
+template <bool DAG, int NT>
+__device__ __noinline__ void slow_site(const HopArgs& a, int p, const char* in, int i, const int* nbr, int flips,
+                                       double2* out) {
+    cplx<double> acc[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc[k] = {0.0, 0.0};
+    const char* Lp = a.links + (size_t)(p * 4) * a.link_block;
+    const char* Lq = a.links + (size_t)((1 - p) * 4) * a.link_block;
+    auto dir = [&](auto dtag) {
+        constexpr int D = decltype(dtag)::value, MU = D >> 1;
+        constexpr bool FWD = (D & 1) == 0;
+        constexpr int S = (FWD == DAG) ? 1 : -1;
+        const int n = nbr[D * NT];
+        cplx<double> s[12], h[6], u[9], uh[6];
+        load_spinor<LQ_F64, double>(in, a.g.Vh, n, s);
+        project<MU, S>(s, h);
+        const int4* lk = reinterpret_cast<const int4*>((FWD ? Lp : Lq) + (size_t)MU * a.link_block);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const int4 v = __ldg(lk + (size_t)k * a.g.Vh + (FWD ? i : n));
+            u[k] = {fix_link_value(v.y, v.x), fix_link_value(v.w, v.z)};
+        }
+        if ((flips >> D) & 1) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) h[k] = cneg(h[k]);
+        }
+        su3_mul<!FWD>(u, h, uh);
+        reconstruct_add<MU, S>(acc, uh);
+    };
+    dir(std::integral_constant<int, 0>());
+    dir(std::integral_constant<int, 1>());
+    dir(std::integral_constant<int, 2>());
+    dir(std::integral_constant<int, 3>());
+    dir(std::integral_constant<int, 4>());
+    dir(std::integral_constant<int, 5>());
+    dir(std::integral_constant<int, 6>());
+    dir(std::integral_constant<int, 7>());
+#pragma unroll
+    for (int k = 0; k < 12; ++k) out[k * NT] = make_double2(acc[k].re, acc[k].im);
+}
+
+// ------------------------------------------------------------------ kernel
+
+constexpr int kFixThreads = 2 * kHopThreads;  // two threads a site
+
+struct FixSmem {
+    static constexpr int PL = 16 * kHopThreads;  // bytes of a plane: 16 a site
+    static constexpr int SPINOR = 0;
+    static constexpr int LINK = 12 * PL;
+    static constexpr int NBR = LINK + 9 * PL;
+    static constexpr int BYTES = NBR + 8 * 4 * kHopThreads;
+};
+
+template <bool DAG, int EPI, bool RED>
+__global__ void __launch_bounds__(kFixThreads, 3) wilson_hop_fixed_kernel(const HopArgs a) {
+    constexpr int NT = kHopThreads, PL = FixSmem::PL;
+    extern __shared__ __align__(16) unsigned char smem[];
+    // lane 16 s + j: spin s of the half spinors of the warp's site j
+    const int spin = (threadIdx.x >> 4) & 1;
+    const int t = (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
+    // grid.x = (rhs, output parity, site tile), rhs fastest (see wilson_hop_kernel)
+    const int rhs = blockIdx.x % a.nrhs;
+    const int pt = blockIdx.x / a.nrhs;
+    const Geom& g = a.g;
+    const int end = a.nsite ? a.site0 + a.nsite : g.Vh;
+    const int i0 = a.site0 + (pt / a.nparity) * NT + t;
+    const bool active = i0 < end;
+    const int i = active ? i0 : end - 1;  // past the end: recomputes the last site, stores nothing
+    const int p = a.parity0 + pt % a.nparity;
+    pdl_enter();
+    if (a.skip && a.skip[(EPI == EPI_DWF ? 0 : rhs) * a.skip_stride]) return;
+
+    const char* __restrict__ in = a.in[p] + (size_t)rhs * a.in_rhs;
+    unsigned char* sp = smem + FixSmem::SPINOR + t * 16;
+    unsigned char* lk = smem + FixSmem::LINK + t * 16;
+    int* nbr = reinterpret_cast<int*>(smem + FixSmem::NBR) + t;  // neighbour of direction d at d NT
+    int flips = 0;                                               // bit d: direction d crosses a boundary with sign -1
+    {
+        int x[4], n[8];
+        cb_coords(g, i, p, x);
+        const int xh = x[0] >> 1;
+        const bool top0 = x[0] + 1 == g.L[0], bot0 = x[0] == 0;
+        n[0] = i - xh + ((top0 ? 0 : x[0] + 1) >> 1);
+        n[1] = i - xh + ((bot0 ? g.L[0] - 1 : x[0] - 1) >> 1);
+        if (g.bc[0] < 0) flips |= (top0 ? 1 : 0) | (bot0 ? 2 : 0);
+        int step = g.Lh0;
+#pragma unroll
+        for (int mu = 1; mu < 4; ++mu) {
+            const bool top = x[mu] == g.L[mu] - 1, bot = x[mu] == 0;
+            n[2 * mu] = top ? i - (g.L[mu] - 1) * step : i + step;
+            n[2 * mu + 1] = bot ? i + (g.L[mu] - 1) * step : i - step;
+            if (g.bc[mu] < 0) flips |= (top ? 1 << (2 * mu) : 0) | (bot ? 2 << (2 * mu) : 0);
+            step *= g.L[mu];
+        }
+        if (spin == 0) {
+#pragma unroll
+            for (int d = 0; d < 8; ++d) nbr[d * NT] = check_site(n[d], g.Vh);
+        }
+    }
+    __syncwarp();
+    const char* __restrict__ links = a.links + (size_t)(p * 4) * a.link_block;
+    const ptrdiff_t other = (p ? -4 : 4) * (ptrdiff_t)a.link_block;  // to the other parity's links
+    const size_t plane = (size_t)g.Vh * 16;
+
+    // the site's two threads copy half of its planes each
+    auto issue_spinor = [&](const char* blk, int site) {
+        const char* src = blk + (size_t)(6 * spin) * plane + (size_t)site * 16;
+        unsigned char* dst = sp + 6 * spin * PL;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) __pipeline_memcpy_async(dst + k * PL, src + k * plane, 16);
+    };
+    auto issue_link = [&](int d) {
+        const bool bwd = d & 1;
+        const char* src = links + (bwd ? other : 0) + (size_t)(d >> 1) * a.link_block + (size_t)(5 * spin) * plane +
+                          (size_t)(bwd ? nbr[d * NT] : i) * 16;
+        unsigned char* dst = lk + 5 * spin * PL;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) __pipeline_memcpy_async(dst + k * PL, src + k * plane, 16);
+        if (spin == 0) __pipeline_memcpy_async(dst + 4 * PL, src + 4 * plane, 16);
+    };
+    // this thread's groups up to the last but one are complete, and so are its partner's
+    auto wait_one = [&]() {
+        __pipeline_wait_prior(1);
+        __syncwarp();
+    };
+
+    // sums over directions, [2 c + {re, im}]: up of spin s; lx and ly of the lower spins, lx (from
+    // x and y hops) of spin 2 + (1 - s), ly (z and t) of spin 2 + s
+    long long up[6], lx[6], ly[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) up[k] = lx[k] = ly[k] = 0;
+    int eb = 0;  // the block's biased exponent: |neighbour components| < 2^(eb - 1022)
+    bool slow = false;
+
+    issue_spinor(in, nbr[NT]);
+    __pipeline_commit();
+    issue_link(1);
+    __pipeline_commit();
+
+    // One body per dimension, run backward, then forward: with one for each of the 8 directions
+    // the SM waited for instructions.  With w_b, w_f the results of the two, a sum that takes
+    // w_f - w_b is formed as sum = w - sum both times.
+    const int sg0 = spin ? 0 : -1, sg1 = ~sg0;  // minus for spin 0 / for spin 1
+    auto dimension = [&](auto mtag) {
+        constexpr int MU = decltype(mtag)::value;
+#pragma unroll 1
+        for (int d = 2 * MU + 1; d >= 2 * MU; --d) {
+            const int bwd = -(d & 1);  // -1: backward, U^dag h = conj(U^T conj(h))
+            const int flip = -((flips >> d) & 1), fim = flip ^ bwd;
+            const int neg = DAG ? bwd : ~bwd;  // -1: projector sign S = -1
+            Fix2 h[6];                         // [2 c + {re, im}] of spin s (backward: of the conjugate)
+            wait_one();
+            {
+                // this spin and the one that the projector adds to it, times i in x and z
+                constexpr bool SW = (MU & 1) == 0;
+                uint2 r[6], q[6];
+                const unsigned char* rp = sp + 3 * spin * PL;
+                const unsigned char* qp = sp + (MU < 2 ? 9 - 3 * spin : 6 + 3 * spin) * PL;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const uint4 v = *reinterpret_cast<const uint4*>(rp + c * PL);
+                    const uint4 x = *reinterpret_cast<const uint4*>(qp + c * PL);
+                    r[2 * c] = make_uint2(v.x, v.y);
+                    r[2 * c + 1] = make_uint2(v.z, v.w);
+                    q[2 * c + (SW ? 1 : 0)] = make_uint2(x.x, x.y);
+                    q[2 * c + (SW ? 0 : 1)] = make_uint2(x.z, x.w);
+                }
+                if constexpr (MU == 3) {
+                    // the time direction is projected in FP64: a ghost spinor rebuilt from its
+                    // spin-projected face (halo.cu) has this half spinor and no other component
+                    // right, and gives the same sums bit for bit.  (The FP64 unit has time for
+                    // these additions; for those of all directions it has not.)
+#pragma unroll
+                    for (int k = 0; k < 6; ++k)
+                        r[k] = words(value(r[k]) + value(make_uint2(q[k].x, q[k].y ^ ((uint32_t)neg << 31))));
+                }
+                float m = 0.f;
+                if constexpr (MU < 3) {
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) m = max_hi(m, r[k].y, q[k].y);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) m = max_hi(m, r[2 * k].y, r[2 * k + 1].y);
+                }
+                m = max_hi(m, __float_as_uint(__shfl_xor_sync(0xffffffffu, m, 16)), 0u);
+                const int e = __float_as_int(m) >> 20;
+                if (e > eb) {  // one bit of headroom: later neighbours seldom move the sums
+                    const int to = max(e + 1, kFixEmin);
+                    const uint32_t n = (uint32_t)(to - eb);
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) {
+                        up[k] = sar64(up[k], n);
+                        lx[k] = sar64(lx[k], n);
+                        ly[k] = sar64(ly[k], n);
+                    }
+                    eb = to;
+                    slow = slow || to > kFixEmax;
+                }
+                const uint32_t e2 = ((uint32_t)max(eb, kFixEmin) << 21) + 0x1fffffu + (5u << 21);
+                // what is added: x: S(im, -re); y: -S (s = 0), S (s = 1); z: as x (s = 0), the
+                // opposite (s = 1)
+                const int tre = flip ^ neg ^ (MU == 1 ? sg0 : MU == 2 ? sg1 : 0);
+                const int tim = fim ^ neg ^ (MU == 0 ? -1 : sg0);
+#pragma unroll
+                for (int k = 0; k < 6; ++k) {
+                    if constexpr (MU == 3) h[k] = fix_one(r[k], e2, k & 1 ? fim : flip);
+                    else h[k] = fix_pair(r[k], q[k], e2, k & 1 ? fim : flip, k & 1 ? tim : tre);
+                }
+            }
+            __syncwarp();  // the site's spinor has been read
+            const int next = bwd ? d - 1 : d + 3;
+            if (MU < 3 || bwd) issue_spinor(in, nbr[next * NT]);
+            else if constexpr (EPI >= EPI_DIAG) issue_spinor(a.x[p] + (size_t)rhs * a.x_rhs, i);
+            __pipeline_commit();
+            wait_one();
+            // w = U h (backward: U^T conj(h), the conjugate of U^dag h), rows of U or U^T
+            long long w[6];
+            const unsigned char* l0 = lk;
+            const unsigned char* l1 = lk + (bwd ? 3 : 1) * PL;
+            const unsigned char* l2 = lk + (bwd ? 6 : 2) * PL;
+            const int sc = (bwd ? 1 : 3) * PL;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const int4 a0 = *reinterpret_cast<const int4*>(l0 + c * sc);
+                const int4 a1 = *reinterpret_cast<const int4*>(l1 + c * sc);
+                const int4 a2 = *reinterpret_cast<const int4*>(l2 + c * sc);
+                const Fix2 u[6] = {{a0.y, a0.x}, {a1.y, a1.x}, {a2.y, a2.x}, {a0.w, a0.z}, {a1.w, a1.z}, {a2.w, a2.z}};
+                const Fix2 x[6] = {h[0], h[2], h[4], {-h[1].hi, -h[1].lo}, {-h[3].hi, -h[3].lo}, {-h[5].hi, -h[5].lo}};
+                const Fix2 y[6] = {h[1], h[3], h[5], h[0], h[2], h[4]};
+                w[2 * c] = fix_dot(u, x);
+                w[2 * c + 1] = fix_dot(u, y);
+            }
+            __syncwarp();  // the site's link has been read
+            if (MU < 3 || bwd) issue_link(next);
+            __pipeline_commit();
+            // sums += [uh; S A_mu^dag uh], uh = w, or conj(w) backward; the lower half as if S > 0
+            // forward (it changes sign at the end otherwise).  Spin s of uh goes, times S, to
+            //   x: i uh of the other lower spin;   y: -uh (s = 0), uh (s = 1) of the other;
+            //   z: i uh (s = 0), -i uh (s = 1) of its own;   t: uh of its own.
+            const long long n = MU == 1 ? (long long)sg0 : (long long)sg1;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const long long re = w[2 * c], im = w[2 * c + 1];
+                up[2 * c] += re;
+                up[2 * c + 1] = im - up[2 * c + 1];
+                if constexpr (MU == 0) {
+                    lx[2 * c] -= im;
+                    lx[2 * c + 1] = re - lx[2 * c + 1];
+                } else if constexpr (MU == 1) {
+                    lx[2 * c] = ((re ^ n) - n) - lx[2 * c];
+                    lx[2 * c + 1] += (im ^ n) - n;
+                } else if constexpr (MU == 2) {
+                    ly[2 * c] -= (im ^ n) - n;
+                    ly[2 * c + 1] = ((re ^ n) - n) - ly[2 * c + 1];
+                } else {
+                    ly[2 * c] = re - ly[2 * c];
+                    ly[2 * c + 1] += im;
+                }
+            }
+        }
+    };
+    dimension(std::integral_constant<int, 0>());
+    dimension(std::integral_constant<int, 1>());
+    dimension(std::integral_constant<int, 2>());
+    dimension(std::integral_constant<int, 3>());
+#pragma unroll
+    for (int k = 0; k < 6; ++k) ly[k] += __shfl_xor_sync(0xffffffffu, lx[k], 16);
+
+    // c_hop, and S of the forward projectors for the lower spins; a power of two (all but the second
+    // hop of the Schur complement) goes into the exponent
+    const double ch = a.c_hop;
+    const uint32_t cw = (uint32_t)__double2hiint(ch);
+    const int ce = (int)((cw >> 20) & 0x7ffu) - 1023;
+    const bool pow2 = (cw & 0xfffffu) == 0 && __double2loint(ch) == 0 && ce >= -64 && ce <= 16;
+    const int ef = eb + (pow2 ? ce : 0);
+    const uint32_t fu = pow2 ? cw : 0u, fl = DAG ? fu : ~fu;
+    double o[12];  // [2 c + {re, im}] of spin s, then of spin 2 + s
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        o[k] = fix_to_double(up[k], ef, fu);
+        o[6 + k] = fix_to_double(ly[k], ef, fl);
+    }
+    if (!pow2) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) o[k] *= ch;
+    }
+    // neighbours that are all zero, subnormal or tiny (the block exponent 0 or held at kFixEmin),
+    // and those out of range above, take the FP64 sums, by way of the site's spinor slot
+    if (__any_sync(0xffffffffu, slow || eb <= kFixEmin)) {
+        const bool mine = slow || eb <= kFixEmin;  // the same for a site's two threads
+        __pipeline_wait_prior(0);
+        __syncwarp();
+        double2* v = reinterpret_cast<double2*>(sp);
+        if (mine && spin == 0) slow_site<DAG, NT>(a, p, in, i, nbr, flips, v);
+        __syncwarp();
+        if (mine) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const double2 b = v[(3 * spin + c) * NT], l = v[(6 + 3 * spin + c) * NT];
+                o[2 * c] = ch * b.x;
+                o[2 * c + 1] = ch * b.y;
+                o[6 + 2 * c] = ch * l.x;
+                o[6 + 2 * c + 1] = ch * l.y;
+            }
+        }
+        __syncwarp();
+        if constexpr (EPI >= EPI_DIAG) issue_spinor(a.x[p] + (size_t)rhs * a.x_rhs, i);
+        __pipeline_commit();
+    }
+    if constexpr (EPI >= EPI_DIAG) {
+        __pipeline_wait_prior(0);
+        __syncwarp();
+        const double cd = a.c_diag;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double2 b = *reinterpret_cast<const double2*>(sp + (3 * spin + c) * PL);
+            const double2 l = *reinterpret_cast<const double2*>(sp + (6 + 3 * spin + c) * PL);
+            o[2 * c] = fma(cd, b.x, o[2 * c]);
+            o[2 * c + 1] = fma(cd, b.y, o[2 * c + 1]);
+            o[6 + 2 * c] = fma(cd, l.x, o[6 + 2 * c]);
+            o[6 + 2 * c + 1] = fma(cd, l.y, o[6 + 2 * c + 1]);
+        }
+    }
+    if constexpr (EPI == EPI_DWF) {
+        const HopShift<double> sh = hop_shift<DAG, double>(a, rhs);
+        const double2* xu = reinterpret_cast<const double2*>(a.x[p] + (size_t)sh.up * a.x_rhs);
+        const double2* xd = reinterpret_cast<const double2*>(a.x[p] + (size_t)sh.dn * a.x_rhs);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double2 b = __ldg(xu + (size_t)(3 * spin + c) * g.Vh + i);
+            const double2 l = __ldg(xd + (size_t)(6 + 3 * spin + c) * g.Vh + i);
+            o[2 * c] = fma(sh.c_up, b.x, o[2 * c]);
+            o[2 * c + 1] = fma(sh.c_up, b.y, o[2 * c + 1]);
+            o[6 + 2 * c] = fma(sh.c_dn, l.x, o[6 + 2 * c]);
+            o[6 + 2 * c + 1] = fma(sh.c_dn, l.y, o[6 + 2 * c + 1]);
+        }
+    }
+    if (active) {
+        double2* out = reinterpret_cast<double2*>(a.out[p] + (size_t)rhs * a.out_rhs);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            out[(size_t)(3 * spin + c) * g.Vh + i] = make_double2(o[2 * c], o[2 * c + 1]);
+            out[(size_t)(6 + 3 * spin + c) * g.Vh + i] = make_double2(o[6 + 2 * c], o[6 + 2 * c + 1]);
+        }
+    }
+    if constexpr (RED) {
+        // a partial for every 32 sites (two warps), group-major (see hop_norm_site)
+        __shared__ double half[kFixThreads / 64];
+        double v = 0;
+        if (active) {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) v = fma(o[k], o[k], v);
+        }
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
+        const int w = threadIdx.x >> 5;
+        if ((w & 1) && (threadIdx.x & 31) == 0) half[w >> 1] = v;
+        __syncthreads();
+        if (!(w & 1) && (threadIdx.x & 31) == 0) {
+            const int wpb = NT >> 5;
+            const int grp = EPI == EPI_DWF ? 0 : rhs;
+            const int nblk = EPI == EPI_DWF ? gridDim.x : gridDim.x / a.nrhs;
+            const int bidx = EPI == EPI_DWF ? blockIdx.x : pt;
+            a.red_partial[(size_t)grp * nblk * wpb + bidx * wpb + (w >> 1)] = v + half[w >> 1];
+        }
+    }
+}
+
+template <bool DAG, int EPI, bool RED>
+cudaError_t launch_fixed_one(const HopArgs& a, cudaStream_t st) {
+    constexpr int NT = kHopThreads, smem = FixSmem::BYTES;
+    auto kern = wilson_hop_fixed_kernel<DAG, EPI, RED>;
+    static bool configured = false;  // attribute set once per process (per instantiation)
+    if (!configured) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        configured = true;
+    }
+    const int nsite = a.nsite ? a.nsite : a.g.Vh;
+    return launch_pdl(kern, dim3(((nsite + NT - 1) / NT) * a.nrhs * a.nparity), dim3(kFixThreads), smem, st, a);
+}
+
+inline cudaError_t launch_hop_fixed(const HopArgs& a, bool dag, int epi, cudaStream_t st) {
+    const bool red = a.red_partial != nullptr;
+    if (red && epi == EPI_HOP) return cudaErrorInvalidValue;
+#define LQ_F_EPI(D)                                                                                    \
+    switch (epi) {                                                                                     \
+    case EPI_HOP: return launch_fixed_one<D, EPI_HOP, false>(a, st);                                   \
+    case EPI_DIAG: return red ? launch_fixed_one<D, EPI_DIAG, true>(a, st)                             \
+                              : launch_fixed_one<D, EPI_DIAG, false>(a, st);                           \
+    default: return red ? launch_fixed_one<D, EPI_DWF, true>(a, st) : launch_fixed_one<D, EPI_DWF, false>(a, st); \
+    }
+    if (dag) { LQ_F_EPI(true) } else { LQ_F_EPI(false) }
+#undef LQ_F_EPI
+}
+
+}  // namespace lq

@@ -402,6 +402,25 @@ __device__ __forceinline__ void store_link(char* __restrict__ blk, int Vh, int i
     }
 }
 
+// A link of the fixed-point FP64 hop (hop_fixed.cuh): plane k of a (parity, mu) block, 16 bytes a
+// site, holds {lo, hi} of the real and of the imaginary part of entry k, v 2^58 = hi 2^30 + lo
+// rounded to nearest, |lo| <= 2^29.
+struct Fix2 {
+    int hi, lo;
+};
+__device__ __forceinline__ Fix2 fix_link_entry(double v) {
+    const long long q = __double2ll_rn(v * 288230376151711744.0);
+    const int hi = (int)((q + (1LL << 29)) >> 30);
+    return {hi, (int)(q - ((long long)hi << 30))};
+}
+__device__ __forceinline__ void store_link_fixed(char* __restrict__ blk, int Vh, int i, const cplx<double> (&u)[9]) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const Fix2 re = fix_link_entry(u[k].re), im = fix_link_entry(u[k].im);
+        reinterpret_cast<int4*>(blk)[(size_t)k * Vh + i] = make_int4(re.lo, re.hi, im.lo, im.hi);
+    }
+}
+
 // ----------------------------------------------- raw (packed) neighbour data
 // The hop issues the loads of the next direction before it computes the
 // current one; holding the data in its packed storage form keeps that

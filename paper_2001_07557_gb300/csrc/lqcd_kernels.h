@@ -36,6 +36,7 @@ struct HopArgs {
     // 1: a launch of at least 8 right-hand sides in FP16/BF16 with 18-real links runs
     // its SU(3) products on the tensor cores (hop_mma.cuh); 0: CUDA cores only
     int mma;
+    int fixed;  // FP64: the links are the fixed-point ones of hop_fixed.cuh
     const int* skip;  // optional per-rhs flags (skip[rhs * skip_stride]): a set flag ends the block at once
     int skip_stride;
     // optional fused |out|^2 per right-hand side (one group for the domain wall):
@@ -121,5 +122,9 @@ cudaError_t link_su3_deviation(int src_prec, const void* src, long nlinks, doubl
 // Gauge links: site-major [site][mu][3][3][2] (F64/F32) -> native [parity][mu] blocks.
 cudaError_t launch_links_to_native(int dst_prec, bool r12, void* dst, int src_prec, const void* src, const Geom& g,
                                    cudaStream_t st);
+// The same for the fixed-point FP64 hop (hop_fixed.cuh).
+cudaError_t launch_links_fixed(void* dst, int src_prec, const void* src, const Geom& g, cudaStream_t st);
+// *bad (device) += the links that the fixed-point hop cannot take (see link_fixed_check_kernel).
+cudaError_t launch_links_fixed_check(int src_prec, const void* src, long nlinks, unsigned* bad, cudaStream_t st);
 
 }  // namespace lq
