@@ -404,6 +404,10 @@ int lq_face_unpack(lq_handle *h, void *dst, int t_dst, const void *wire, int fmt
  *     (LQ_ERR_LAYOUT otherwise).  The caller owns all three.
  *   - C may be the same pointer as A or as B (the product is formed in place
  *     tile by tile); any other overlap is LQ_ERR_ARG.
+ *   - FP64 matrices of the scale of SU(3) (every real at most 1, every row of A
+ *     and column of B with a real of at least 1/4) are multiplied in 64-bit fixed
+ *     point: an entry is a sum good to 2^-57, rounded to FP64 once.  Others are
+ *     multiplied in FP64, FP32 ones in FP32.
  *   - n = 0 is a no-op; n < 0 or a null pointer with n > 0 is LQ_ERR_ARG.
  *   - Asynchronous on `stream`.  No handle is needed and nothing is allocated.
  * Tiles of A and B move to shared memory by bulk asynchronous copies that

@@ -20,8 +20,8 @@
 //
 // Precision: the sums carry 57 bits below the largest neighbour component (56 where the
 // headroom of the block exponent is used), against the 53 bits of each FP64 partial sum.
-// Against 64-bit reference results of D on 32^4 the error is 1.1e-16 (FP64 kernel 1.2e-16),
-// of Mhat^dag on 10x14x18x22 0.96e-16 (1.1e-16).  What is not finite, beyond 2^976 or below
+// Against sums in quadruple precision the hop on 8^4 (random and smooth links) is 5.8e-17 off,
+// norm-wise, and 1.5e-16 with the FP64 kernel.  What is not finite, beyond 2^976 or below
 // 2^-894 takes the FP64 sums of slow_site.
 //
 // It needs links with |u| <= 1 and rows and columns of 1-norm <= 2.75 (SU(3): <= 2.45), which
@@ -44,98 +44,13 @@
 
 #include <cuda_pipeline.h>
 
+#include "fixed.cuh"
 #include "hop.cuh"
 
 namespace lq {
 
 constexpr int kFixEmin = 128;    // biased exponents the block may have
 constexpr int kFixEmax = 2000;
-constexpr uint32_t kFixMask = (1u << 30) - 1;
-
-__device__ __forceinline__ uint64_t shr64(uint64_t v, uint32_t n) {  // 0 for n > 63
-    uint64_t r;
-    asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
-    return r;
-}
-__device__ __forceinline__ uint32_t shr32(uint32_t v, uint32_t n) {  // 0 for n > 31
-    uint32_t r;
-    asm("shr.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
-    return r;
-}
-__device__ __forceinline__ long long sar64(long long v, uint32_t n) {  // the sign for n > 63
-    long long r;
-    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
-    return r;
-}
-__device__ __forceinline__ long long mad_wide(int a, int b, long long c) { return (long long)a * b + c; }
-
-__device__ __forceinline__ double value(uint2 w) { return __hiloint2double((int)w.y, (int)w.x); }
-__device__ __forceinline__ uint2 words(double v) {
-    return make_uint2((unsigned)__double2loint(v), (unsigned)__double2hiint(v));
-}
-
-// The larger of m and the high words of two doubles without their signs, compared as FP32
-// numbers (of the same order; a word that is an FP32 NaN, from 2^1017 up, gives a NaN, which is
-// above every exponent allowed).
-__device__ __forceinline__ float max_hi(float m, uint32_t a, uint32_t b) {
-    float r;
-    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(fabsf(__uint_as_float(a))), "f"(fabsf(__uint_as_float(b))));
-    return r;
-}
-
-// |x| as fixed point below the block exponent (rounded toward zero), and the sign as +-1
-struct FixMag {
-    int hi, lo, s;
-};
-// e2 = 2 (Eb 2^20 + 2^20 - 1) + 1 + 5 2^21 with Eb the block's biased exponent: e2 - 2 w
-// (w: the high word of x) has Eb - e + 5 in its top 11 bits whatever x's sign and mantissa
-// are.  neg = 0, or -1 to negate.  A zero or subnormal x is shifted out, for Eb >= kFixEmin.
-__device__ __forceinline__ FixMag fix_mag(uint2 x, uint32_t e2, int neg) {
-    const uint32_t w = x.y, l = x.x;
-    const uint32_t d = (e2 - 2u * w) >> 21;  // the block exponent above x's, plus 5
-    const uint32_t nh = __funnelshift_l(l, w, 11) | 0x80000000u, nl = l << 11;  // mantissa, top bit set
-    FixMag f;
-    f.lo = (int)((uint32_t)shr64(((uint64_t)nh << 32) | nl, d) & kFixMask);
-    f.hi = (int)shr32(nh, d - 2u);
-    f.s = (((int)w >> 31) ^ neg) | 1;
-    return f;
-}
-__device__ __forceinline__ Fix2 fix_one(uint2 x, uint32_t e2, int neg) {
-    const FixMag f = fix_mag(x, e2, neg);
-    return {f.hi * f.s, f.lo * f.s};
-}
-__device__ __forceinline__ Fix2 fix_pair(uint2 x, uint2 y, uint32_t e2, int nx, int ny) {
-    const FixMag f = fix_mag(x, e2, nx), g = fix_mag(y, e2, ny);
-    return {f.hi * f.s + g.hi * g.s, f.lo * f.s + g.lo * g.s};
-}
-
-// sum_k x_k y_k over six products, rounded to units of 2^60 of the product of the scales
-__device__ __forceinline__ long long fix_dot(const Fix2 (&u)[6], const Fix2 (&h)[6]) {
-    long long mid = 1LL << 29, top;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        mid = mad_wide(u[k].hi, h[k].lo, mid);
-        mid = mad_wide(u[k].lo, h[k].hi, mid);
-    }
-    top = mid >> 30;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) top = mad_wide(u[k].hi, h[k].hi, top);
-    return top;
-}
-
-// v 2^(eb - 1079) rounded to nearest, eb a biased exponent in range; negated for the high bit of flip
-__device__ __forceinline__ double fix_to_double(long long v, int eb, uint32_t flip) {
-    const uint32_t sign = ((uint32_t)(v >> 32) ^ flip) & 0x80000000u;
-    uint64_t m = (uint64_t)(v < 0 ? -v : v);
-    int lz = __clz((int)(m >> 32));
-    if (lz == 32) {  // rare: cancelled by 2^-30
-        if (m == 0) return 0.0;
-        lz += __clz((int)(uint32_t)m);
-    }
-    m <<= lz;
-    const uint64_t b = (m >> 11) + ((m >> 10) & 1);  // the leading bit carries into the exponent
-    return __hiloint2double((int)(((uint32_t)(b >> 32) + ((uint32_t)(eb + 6 - lz) << 20)) | sign), (int)(uint32_t)b);
-}
 
 // ------------------------------------------------------------------- links
 

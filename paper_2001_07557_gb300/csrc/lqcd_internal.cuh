@@ -19,6 +19,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "fixed.cuh"
 #include "lqcd.h"
 
 namespace lq {
@@ -405,9 +406,6 @@ __device__ __forceinline__ void store_link(char* __restrict__ blk, int Vh, int i
 // A link of the fixed-point FP64 hop (hop_fixed.cuh): plane k of a (parity, mu) block, 16 bytes a
 // site, holds {lo, hi} of the real and of the imaginary part of entry k, v 2^58 = hi 2^30 + lo
 // rounded to nearest, |lo| <= 2^29.
-struct Fix2 {
-    int hi, lo;
-};
 __device__ __forceinline__ Fix2 fix_link_entry(double v) {
     const long long q = __double2ll_rn(v * 288230376151711744.0);
     const int hi = (int)((q + (1LL << 29)) >> 30);

@@ -13,8 +13,9 @@
 //   * the products go to one of two output buffers, which one thread writes
 //     back with a bulk store.
 // FP32 is bound by HBM bandwidth (216 bytes and 198 flop per matrix).  FP64
-// is bound by the FP64 units: 198 flop take longer at GB300's FP64 rate than
-// its 432 bytes take to move.  Every barrier wait is bounded; a wait that runs
+// would be bound by the FP64 units: 198 flop take longer at GB300's FP64 rate
+// than its 432 bytes take to move.  Matrices of SU(3) scale are therefore
+// multiplied in fixed point on the integer units.  Every barrier wait is bounded; a wait that runs
 // out is counted in g_wait_timeouts and its block stops.  Before it returns,
 // the block waits (bounded again) for the copies it issued into its other
 // stage, and for its bulk stores, so that no copy into its shared memory is
@@ -26,6 +27,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "fixed.cuh"
 #include "lqcd.h"
 #include "trace.h"
 
@@ -114,26 +116,83 @@ __device__ __forceinline__ void su3_product(const T2 (&a)[9], const T2 (&b)[9], 
     }
 }
 
+// The FP64 product in fixed point (fixed.cuh), for two matrices whose scale is that of SU(3):
+// every real at most 1 (and 2^-20), every row of A and column of B with a real of at least 1/4,
+// as unitary ones have (1/sqrt 6).  The block exponent is then the same for all, 2^0, and an
+// entry of C is rounded once from a sum exact to 2^-57.  False for any other pair, which the
+// FP64 unit multiplies.  Against sums in quadruple precision the products of smooth links
+// (exp(0.3 i H)) are 3.9e-17 off, norm-wise, and 7.4e-17 with the FP64 unit.  108 FP64 instructions
+// at 77 clocks a warp and SM sub-partition compare with about 1,400 integer ones here.  48^4: 991 us in FP64, 511 us with two blocks an SM and
+// output buffers, 418 us with three blocks and in place (0.81 of the HBM time of its bytes;
+// four blocks of one stage 434 us).
+__device__ __forceinline__ bool su3_product_fixed(const double2* a, const double2* b, double2 (&c)[9]) {
+    constexpr int EB = 1022;
+    constexpr uint32_t E2 = ((uint32_t)EB << 21) + 0x1fffffu + (5u << 21);
+    constexpr int kOne = 0x3ff00001, kQuarter = 0x3fd00000;
+    Fix2 fa[18];
+    int top = 0, low = 0x7fffffff;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        float m = 0.f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint2 re = words(a[3 * i + k].x), im = words(a[3 * i + k].y);
+            m = max_hi(m, re.y, im.y);
+            fa[6 * i + k] = fix_one(re, E2, 0);
+            fa[6 * i + 3 + k] = fix_one(im, E2, 0);
+        }
+        top = max(top, __float_as_int(m));
+        low = min(low, __float_as_int(m));
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        float m = 0.f;
+        Fix2 x[6], y[6];  // column j as the factors of the real and of the imaginary part
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint2 re = words(b[3 * k + j].x), im = words(b[3 * k + j].y);
+            m = max_hi(m, re.y, im.y);
+            x[k] = y[3 + k] = fix_one(re, E2, 0);
+            y[k] = fix_one(im, E2, 0);
+            x[3 + k] = {-y[k].hi, -y[k].lo};
+        }
+        top = max(top, __float_as_int(m));
+        low = min(low, __float_as_int(m));
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const Fix2 u[6] = {fa[6 * i], fa[6 * i + 1], fa[6 * i + 2], fa[6 * i + 3], fa[6 * i + 4], fa[6 * i + 5]};
+            // units of 2^60 / 2^118 = 2^-58
+            c[3 * i + j] = make_double2(fix_to_double(fix_dot(u, x), 1021, 0u), fix_to_double(fix_dot(u, y), 1021, 0u));
+        }
+    }
+    return top <= kOne && low >= kQuarter;
+}
+
 // Shared memory: stage s holds the tile of A at 2*s*TB and of B at (2*s+1)*TB,
-// output buffer o at (4+o)*TB, the two stage barriers at 6*TB.
+// output buffer o at (4+o)*TB, the two stage barriers after them.  FP64 has no output
+// buffers: a thread writes its product over its own matrix of A, and the stage is filled
+// again once the store has read it.  That leaves room for 3 blocks an SM instead of 2,
+// which the integer product needs to hide its latencies (see su3_product_fixed).
 template <typename T, int TS>
 struct Su3Cfg {
     using T2 = typename Cx2<T>::type;
+    static constexpr bool IN_PLACE = sizeof(T) == 8;
     static constexpr int MB = 9 * (int)sizeof(T2);  // bytes per matrix
     static constexpr int TB = TS * MB;              // bytes per tile
-    static constexpr int SMEM = 6 * TB + 16;
+    static constexpr int BARS = (IN_PLACE ? 4 : 6) * TB;
+    static constexpr int SMEM = BARS + 16;
 };
 
 // stall != 0 (testing only) arms each stage barrier for 16 more bytes than its
 // copies bring, so that the bounded wait runs out.
 template <typename T, int TS>
-__global__ void __launch_bounds__(TS) su3_mul_kernel(const char* A, const char* B, char* C, long n, int stall) {
+__global__ void __launch_bounds__(TS, sizeof(T) == 8 ? 3 : 1) su3_mul_kernel(const char* A, const char* B, char* C, long n, int stall) {
     using Cfg = Su3Cfg<T, TS>;
     using T2 = typename Cfg::T2;
     constexpr int MB = Cfg::MB, TB = Cfg::TB;
     extern __shared__ __align__(128) unsigned char sm[];
     __shared__ int s_ok;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + 6 * TB);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + Cfg::BARS);
     const int t = threadIdx.x;
     const long ntiles = (n + TS - 1) / TS;
     // matrices of a tile, and those moved by the bulk copies: a bulk copy moves a
@@ -175,19 +234,24 @@ __global__ void __launch_bounds__(TS) su3_mul_kernel(const char* A, const char* 
             break;
         }
         const int cnt = count(tile), nb = bulk(cnt);
-        unsigned char* cbuf = sm + (4 + (it & 1)) * TB;
+        unsigned char* cbuf = sm + (Cfg::IN_PLACE ? 2 * s : 4 + (it & 1)) * TB;
         if (t < cnt) {
-            T2 a[9], b[9], c[9];
+            T2 c[9];
             const T2* pa = t < nb ? reinterpret_cast<const T2*>(sm + 2 * s * TB + t * MB)
                                   : reinterpret_cast<const T2*>(A + (tile * TS + t) * MB);
             const T2* pb = t < nb ? reinterpret_cast<const T2*>(sm + (2 * s + 1) * TB + t * MB)
                                   : reinterpret_cast<const T2*>(B + (tile * TS + t) * MB);
+            bool done = false;
+            if constexpr (sizeof(T) == 8) done = su3_product_fixed(pa, pb, c);
+            if (!done) {
+                T2 a[9], b[9];
 #pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                a[k] = pa[k];
-                b[k] = pb[k];
+                for (int k = 0; k < 9; ++k) {
+                    a[k] = pa[k];
+                    b[k] = pb[k];
+                }
+                su3_product(a, b, c);
             }
-            su3_product(a, b, c);
             T2* pc = t < nb ? reinterpret_cast<T2*>(cbuf + t * MB) : reinterpret_cast<T2*>(C + (tile * TS + t) * MB);
 #pragma unroll
             for (int k = 0; k < 9; ++k) pc[k] = c[k];
@@ -198,9 +262,10 @@ __global__ void __launch_bounds__(TS) su3_mul_kernel(const char* A, const char* 
             if (nb) bulk_store(C + tile * TB, smem_u32(cbuf), (uint32_t)nb * MB);
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             const long next = tile + 2L * gridDim.x;
+            if (Cfg::IN_PLACE) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             if (next < ntiles) issue(next, s);
             // the store issued one iteration ago has read the buffer the next iteration fills
-            asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            if (!Cfg::IN_PLACE) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
         }
     }
     if (t == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
