@@ -13,35 +13,23 @@ namespace lq {
 
 namespace {
 
-template <int SP>
-__device__ __forceinline__ void load_sm(const void* base, size_t site, cplx<double> (&s)[12]) {
+template <int SP, typename T>
+__device__ __forceinline__ void load_sm(const void* base, size_t site, cplx<T> (&s)[12]) {
     if constexpr (SP == LQ_F64) {
         const double2* q = reinterpret_cast<const double2*>(base) + site * 12;
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
             double2 v = q[k];
-            s[k] = {v.x, v.y};
+            s[k] = {(T)v.x, (T)v.y};
         }
     } else {
-        const float2* q = reinterpret_cast<const float2*>(base) + site * 12;
+        const float4* q = reinterpret_cast<const float4*>(base) + site * 6;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            float2 v = q[k];
-            s[k] = {(double)v.x, (double)v.y};
+        for (int k = 0; k < 6; ++k) {
+            float4 v = q[k];
+            s[2 * k] = {(T)v.x, (T)v.y};
+            s[2 * k + 1] = {(T)v.z, (T)v.w};
         }
-    }
-}
-
-template <int SP>
-__device__ __forceinline__ void store_sm(void* base, size_t site, const cplx<double> (&s)[12]) {
-    if constexpr (SP == LQ_F64) {
-        double2* q = reinterpret_cast<double2*>(base) + site * 12;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) q[k] = make_double2(s[k].re, s[k].im);
-    } else {
-        float2* q = reinterpret_cast<float2*>(base) + site * 12;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) q[k] = make_float2((float)s[k].re, (float)s[k].im);
     }
 }
 
@@ -51,9 +39,18 @@ __device__ __forceinline__ size_t lexi_of(const Geom& g, int cb, int p) {
     return (size_t)x[0] + (size_t)g.L[0] * (x[1] + (size_t)g.L[1] * (x[2] + (size_t)g.L[2] * x[3]));
 }
 
+constexpr int kBlock = 128;
+
+// Arithmetic of a conversion: FP64 only where both sides are FP64 or one is and the other holds
+// FP32 values to widen or round; FP32 otherwise (FP32 -> FP64 -> FP32 costs two conversions a real
+// on the FP64 unit and changes nothing).
+template <int DP, int SP>
+using ConvT = typename std::conditional<DP == LQ_F64 || SP == LQ_F64, double, float>::type;
+
 // grid.y = rhs * nparity + parity index
-template <int DP, int SP, bool TO_NATIVE>
-__global__ void spinor_layout_kernel(char* nat, void* sm, Geom g, bool full, int parity, int nparity) {
+template <int DP, int SP>
+__global__ void __launch_bounds__(kBlock) spinor_to_native_kernel(char* nat, const void* sm, Geom g, bool full,
+                                                                  int parity, int nparity) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.Vh) return;
     const int pi = blockIdx.y % nparity;
@@ -62,13 +59,52 @@ __global__ void spinor_layout_kernel(char* nat, void* sm, Geom g, bool full, int
     const size_t nsites_sm = full ? 2 * (size_t)g.Vh : (size_t)g.Vh;
     const size_t site = (size_t)rhs * nsites_sm + (full ? lexi_of(g, i, p) : (size_t)i);
     char* blk = nat + ((size_t)rhs * nparity + pi) * (size_t)spinor_site_bytes(DP) * g.Vh;
-    cplx<double> s[12];
-    if constexpr (TO_NATIVE) {
-        load_sm<SP>(sm, site, s);
-        store_spinor<DP, double>(blk, g.Vh, i, s);
-    } else {
-        load_spinor<DP, double>(blk, g.Vh, i, s);
-        store_sm<SP>(sm, site, s);
+    cplx<ConvT<DP, SP>> s[12];
+    load_sm<SP>(sm, site, s);
+    store_spinor<DP>(blk, g.Vh, i, s);
+}
+
+// The site-major side is written through shared memory, so that a warp's stores cover whole
+// sites (192 or 96 consecutive bytes): a thread that wrote its own site put 16 bytes into each of
+// 32 lines with every store (32^4, FP64: 182 us for 403 MB, here 82 us; FP32 to FP32 88 and 41 us).
+// A site's slot is 16 bytes longer than the site, which keeps both sides free of bank conflicts.
+template <int NP, int SP>
+__global__ void __launch_bounds__(kBlock) spinor_from_native_kernel(void* sm, const char* nat, Geom g, bool full,
+                                                                    int parity, int nparity) {
+    using T = ConvT<NP, SP>;
+    constexpr int CH = SP == LQ_F64 ? 12 : 6;  // 16-byte chunks of a site
+    constexpr int PITCH = CH + 1;
+    __shared__ uint4 slots[kBlock * PITCH];
+    __shared__ size_t where[kBlock];
+    const int t = threadIdx.x, w = t & ~31, lane = t & 31;
+    const int i = blockIdx.x * kBlock + t;
+    const int pi = blockIdx.y % nparity;
+    const int rhs = blockIdx.y / nparity;
+    const int p = full ? pi : parity;
+    if (blockIdx.x * kBlock + w >= g.Vh) return;  // the warp's first site
+    if (i < g.Vh) {
+        const size_t nsites_sm = full ? 2 * (size_t)g.Vh : (size_t)g.Vh;
+        where[t] = (size_t)rhs * nsites_sm + (full ? lexi_of(g, i, p) : (size_t)i);
+        cplx<T> s[12];
+        load_spinor<NP>(nat + ((size_t)rhs * nparity + pi) * (size_t)spinor_site_bytes(NP) * g.Vh, g.Vh, i, s);
+        if constexpr (SP == LQ_F64) {
+            double2* q = reinterpret_cast<double2*>(slots + t * PITCH);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) q[k] = make_double2(s[k].re, s[k].im);
+        } else {
+            float4* q = reinterpret_cast<float4*>(slots + t * PITCH);
+#pragma unroll
+            for (int k = 0; k < 6; ++k)
+                q[k] = make_float4((float)s[2 * k].re, (float)s[2 * k].im, (float)s[2 * k + 1].re,
+                                   (float)s[2 * k + 1].im);
+        }
+    }
+    __syncwarp();
+    const int sites = min(32, g.Vh - (int)blockIdx.x * kBlock - w);
+#pragma unroll
+    for (int k = 0; k < CH; ++k) {
+        const int c = k * 32 + lane, j = c / CH, part = c - j * CH;
+        if (j < sites) reinterpret_cast<uint4*>(sm)[where[w + j] * CH + part] = slots[(w + j) * PITCH + part];
     }
 }
 
@@ -114,8 +150,6 @@ __global__ void links_kernel(char* dst, const void* src, Geom g, size_t link_blo
         else store_link<DP, R12>(dst + (size_t)(p * 4 + mu) * link_block, g.Vh, i, u);
     }
 }
-
-constexpr int kBlock = 128;
 
 // Largest deviation of a link from SU(3): max over the entries of |U^dag U - 1|
 // and |det U - 1|, in FP64.  Two-row compression rebuilds row 3 as
@@ -221,11 +255,10 @@ cudaError_t launch_spinor_to_native(int dst_prec, void* dst, int src_prec, const
     const int np = full ? 2 : 1;
     dim3 grid((g.Vh + kBlock - 1) / kBlock, nrhs * np);
     char* d = static_cast<char*>(dst);
-    void* s = const_cast<void*>(src);
     if (src_prec == LQ_F64) {
-        LQ_DP_SWITCH(dst_prec, (spinor_layout_kernel<DP, LQ_F64, true><<<grid, kBlock, 0, st>>>(d, s, g, full, parity, np)))
+        LQ_DP_SWITCH(dst_prec, (spinor_to_native_kernel<DP, LQ_F64><<<grid, kBlock, 0, st>>>(d, src, g, full, parity, np)))
     } else {
-        LQ_DP_SWITCH(dst_prec, (spinor_layout_kernel<DP, LQ_F32, true><<<grid, kBlock, 0, st>>>(d, s, g, full, parity, np)))
+        LQ_DP_SWITCH(dst_prec, (spinor_to_native_kernel<DP, LQ_F32><<<grid, kBlock, 0, st>>>(d, src, g, full, parity, np)))
     }
     return cudaGetLastError();
 }
@@ -234,11 +267,11 @@ cudaError_t launch_spinor_from_native(int dst_prec, void* dst, int src_prec, con
                                       bool full, int parity, int nrhs, cudaStream_t st) {
     const int np = full ? 2 : 1;
     dim3 grid((g.Vh + kBlock - 1) / kBlock, nrhs * np);
-    char* n = const_cast<char*>(static_cast<const char*>(src));
+    const char* n = static_cast<const char*>(src);
     if (dst_prec == LQ_F64) {
-        LQ_DP_SWITCH(src_prec, (spinor_layout_kernel<DP, LQ_F64, false><<<grid, kBlock, 0, st>>>(n, dst, g, full, parity, np)))
+        LQ_DP_SWITCH(src_prec, (spinor_from_native_kernel<DP, LQ_F64><<<grid, kBlock, 0, st>>>(dst, n, g, full, parity, np)))
     } else {
-        LQ_DP_SWITCH(src_prec, (spinor_layout_kernel<DP, LQ_F32, false><<<grid, kBlock, 0, st>>>(n, dst, g, full, parity, np)))
+        LQ_DP_SWITCH(src_prec, (spinor_from_native_kernel<DP, LQ_F32><<<grid, kBlock, 0, st>>>(dst, n, g, full, parity, np)))
     }
     return cudaGetLastError();
 }
