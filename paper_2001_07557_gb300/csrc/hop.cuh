@@ -30,26 +30,7 @@ __device__ __forceinline__ void hop_add_diag(const HopArgs& a, const cplx<T> (&x
     }
 }
 
-// c_shift (S x)(s): P+ = upper spins (gamma_5 = diag(1,1,-1,-1)).  Non-dagger: upper from
-// s-1, lower from s+1; dagger swaps.  Coefficient c_shift (Shamir: -1), times -mf across the wall.
-template <typename T>
-struct HopShift {
-    int up, dn;     // slices that the upper and the lower spins come from
-    T c_up, c_dn;
-};
-template <bool DAG, typename T>
-__device__ __forceinline__ HopShift<T> hop_shift(const HopArgs& a, int s) {
-    const int Ls = a.Ls;
-    const bool first = s == 0, last = s + 1 == Ls;
-    const int below = first ? Ls - 1 : s - 1, above = last ? 0 : s + 1;
-    const T c = (T)a.c_shift, cw = (T)(-a.c_shift * a.mf);
-    HopShift<T> h;
-    h.up = DAG ? above : below;
-    h.dn = DAG ? below : above;
-    h.c_up = (DAG ? last : first) ? cw : c;
-    h.c_dn = (DAG ? first : last) ? cw : c;
-    return h;
-}
+// o += c_shift (S x)(s)
 template <int P, bool DAG, typename T>
 __device__ __forceinline__ void hop_add_shift(const HopArgs& a, int s, int p, int i, cplx<T> (&o)[12]) {
     const HopShift<T> h = hop_shift<DAG, T>(a, s);

@@ -19,8 +19,11 @@
 //     current one, and the first ones overlap the staging of the links.
 // Per site and right-hand side the L2 traffic drops from 8 neighbours + 8
 // links to 8 neighbours + 8/N links (24^3 x 48, 12 right-hand sides, FP32:
-// 14.1 -> 8.8 GB per launch).  Measured, FP16/BF16 storage (whose hops are
-// issue-bound) do not gain from it and keep the hop_async.cuh kernel.
+// 14.1 -> 8.8 GB per launch).  FP16/BF16 storage with three-row links (whose
+// hops are issue-bound) does not gain from it and keeps the hop_async.cuh kernel;
+// with two-row links it does, because the third rows are rebuilt (and all links
+// converted to FP32) once and not for every right-hand side: 24^3 x 48, 12 FP16
+// ones 524 -> 421 us.
 // The arithmetic per site and right-hand side is that of hop_async.cuh, in the
 // same order, so a right-hand side comes out bit for bit as it does from a
 // launch of its own; the fused-norm partials fill the same slots with the same
@@ -35,18 +38,25 @@ namespace lq {
 
 // Block shape, measured on 24^3 x 48 with 12 right-hand sides (FP32) and on the
 // 16^4 x 16 domain wall: 32 sites x 4 groups with five resident blocks of 128
-// threads (102 registers, 43 KB of shared memory each) 494 / 72 us; 64 x 4 with
+// threads (96 registers, 43 KB of shared memory each) 494 / 72 us; 64 x 4 with
 // two blocks of 256 threads (128 registers) 527 / 76 us; 64 x 3 with three
-// blocks 533 / 86 us; 32 x 8 with three blocks 606 / 84 us.
+// blocks 533 / 86 us; 32 x 8 with three blocks 606 / 84 us.  FP16 with two-row
+// links: four blocks 455 us, five 432, six (80 registers) 421.
 constexpr int kShSites = 32;     // sites per tile (one warp of each group)
-constexpr int kShGroups = 4;     // groups of threads per block, each taking every kShGroups-th right-hand side
-constexpr int kShMinBlocks = 5;  // resident blocks per SM the register budget is set for
+constexpr int kShGroups = 4;     // groups of threads per block at most, group g taking every G-th right-hand side
+// resident blocks per SM the register budget is set for
+template <int P, int G>
+constexpr int shared_min_blocks() {
+    return (P == LQ_F32 ? 20 : 24) / G;
+}
 
 // The tile's links in shared memory: per direction, LinkLayout's 16-byte
 // chunks chunk-major over the tile's sites, then the tail chunk.
+// Two-row 16-bit links are staged as 18 FP32 reals, rebuilt once for all right-hand sides.
 template <int P, bool R12>
 struct LinkTile {
-    using LL = LinkLayout<P, R12>;
+    static constexpr bool REBUILD = Prec<P>::has_norm && R12;
+    using LL = LinkLayout<REBUILD ? LQ_F32 : P, R12 && !REBUILD>;
     static constexpr int NS = kShSites;
     static constexpr int DIR = (LL::NFULL * 16 + LL::TAIL) * NS;
     static constexpr int BYTES = 8 * DIR;
@@ -55,21 +65,33 @@ struct LinkTile {
 template <int P, bool R12>
 __device__ __forceinline__ void tile_link_stage(unsigned char* dir, const char* __restrict__ blk, int Vh, int site,
                                                 int s) {
-    using LL = LinkLayout<P, R12>;
+    using LL = typename LinkTile<P, R12>::LL;
     constexpr int NS = kShSites;
+    if constexpr (LinkTile<P, R12>::REBUILD) {
+        cplx<float> u[9];
+        load_link<P, true, float>(blk, Vh, site, u);
+        float4* q = reinterpret_cast<float4*>(dir) + s;
 #pragma unroll
-    for (int c = 0; c < LL::NFULL; ++c)
-        __pipeline_memcpy_async(dir + (c * NS + s) * 16, blk + ((size_t)c * Vh + site) * 16, 16);
-    if constexpr (LL::TAIL > 0)
-        __pipeline_memcpy_async(dir + LL::NFULL * 16 * NS + s * LL::TAIL,
-                                blk + (size_t)LL::NFULL * 16 * Vh + (size_t)site * LL::TAIL, LL::TAIL);
+        for (int c = 0; c < 4; ++c) q[c * NS] = make_float4(u[2 * c].re, u[2 * c].im, u[2 * c + 1].re, u[2 * c + 1].im);
+        reinterpret_cast<float2*>(dir + 64 * NS)[s] = make_float2(u[8].re, u[8].im);
+    } else {
+#pragma unroll
+        for (int c = 0; c < LL::NFULL; ++c)
+            __pipeline_memcpy_async(dir + (c * NS + s) * 16, blk + ((size_t)c * Vh + site) * 16, 16);
+        if constexpr (LL::TAIL > 0)
+            __pipeline_memcpy_async(dir + LL::NFULL * 16 * NS + s * LL::TAIL,
+                                    blk + (size_t)LL::NFULL * 16 * Vh + (size_t)site * LL::TAIL, LL::TAIL);
+    }
 }
 
+// a staged link
 template <int P, bool R12>
 __device__ __forceinline__ void tile_link(const unsigned char* dir, int s, cplx<float> (&u)[9]) {
-    using LL = LinkLayout<P, R12>;
+    using LL = typename LinkTile<P, R12>::LL;
+    constexpr bool TWO = R12 && !LinkTile<P, R12>::REBUILD;  // still two rows
     constexpr int NS = kShSites;
-    RawLink<P, R12> r;
+    RawLink<LQ_F32, TWO> r;
+    static_assert(LL::NFULL == LinkLayout<LQ_F32, TWO>::NFULL, "links are staged in FP32");
 #pragma unroll
     for (int c = 0; c < LL::NFULL; ++c) {
         const uint4 v = *reinterpret_cast<const uint4*>(dir + (c * NS + s) * 16);
@@ -78,15 +100,12 @@ __device__ __forceinline__ void tile_link(const unsigned char* dir, int s, cplx<
         r.w[4 * c + 2] = v.z;
         r.w[4 * c + 3] = v.w;
     }
-    const unsigned char* tail = dir + LL::NFULL * 16 * NS;
     if constexpr (LL::TAIL == 8) {
-        const uint2 v = *reinterpret_cast<const uint2*>(tail + s * 8);
+        const uint2 v = *reinterpret_cast<const uint2*>(dir + LL::NFULL * 16 * NS + s * 8);
         r.w[4 * LL::NFULL] = v.x;
         r.w[4 * LL::NFULL + 1] = v.y;
-    } else if constexpr (LL::TAIL == 4) {
-        r.w[4 * LL::NFULL] = *reinterpret_cast<const uint32_t*>(tail + s * 4);
     }
-    raw_unpack<P, R12, float>(r, u);
+    raw_unpack<LQ_F32, TWO, float>(r, u);
 }
 
 template <int P, bool R12, int NT, int S>
@@ -105,8 +124,8 @@ __device__ __forceinline__ size_t shared_red_slot(const HopArgs& a, int epi_dwf,
 }
 
 template <int P, bool R12, bool DAG, int EPI, int G, int S, bool RED>
-__global__ void __launch_bounds__(kShSites* G, kShMinBlocks) wilson_hop_shared_kernel(const HopArgs a) {
-    static_assert(!Prec<P>::has_norm, "the shared-link hop serves FP32 storage");
+__global__ void __launch_bounds__(kShSites* G, shared_min_blocks<P, G>()) wilson_hop_shared_kernel(const HopArgs a) {
+    static_assert(!Prec<P>::has_norm || R12, "the shared-link hop serves FP32 storage and two-row 16-bit links");
     static_assert(kShSites % 32 == 0, "a warp must hold sites of one group (one right-hand side)");
     constexpr int NS = kShSites, NT = NS * G;
     using T = float;
@@ -227,11 +246,17 @@ __global__ void __launch_bounds__(kShSites* G, kShMinBlocks) wilson_hop_shared_k
         smem_spinor<P, R12, NT>(st, t, sp, nrm);                                      \
         project<MU, SG>(sp, h);                                                       \
         tile_link<P, R12>(links + (D)*LT::DIR, s, u);                                 \
-        if (FWD ? sf[MU] : sb[MU]) {                                                  \
-            _Pragma("unroll") for (int k = 0; k < 6; ++k) h[k] = cneg(h[k]);          \
+        const bool sgn = FWD ? sf[MU] : sb[MU];                                       \
+        if constexpr (Prec<P>::has_norm) {                                            \
+            su3_mul<!FWD>(u, h, uh);                                                  \
+            reconstruct_fma<MU, SG>(acc, uh, sgn ? -nrm : nrm);                       \
+        } else {                                                                      \
+            if (sgn) {                                                                \
+                _Pragma("unroll") for (int k = 0; k < 6; ++k) h[k] = cneg(h[k]);      \
+            }                                                                         \
+            su3_mul<!FWD>(u, h, uh);                                                  \
+            reconstruct_add<MU, SG>(acc, uh);                                         \
         }                                                                             \
-        su3_mul<!FWD>(u, h, uh);                                                      \
-        reconstruct_add<MU, SG>(acc, uh);                                             \
         if (++slot == S) slot = 0;                                                    \
     }
         LQ_SH_DIR(0)
@@ -312,9 +337,9 @@ __global__ void __launch_bounds__(kShSites* G, kShMinBlocks) wilson_hop_shared_k
 // whose larger shared-memory carve-out leaves less L1 for the epilogue's reads.
 constexpr int kSharedStages = 2;
 
-template <int P, bool R12, bool DAG, int EPI, bool RED>
+template <int P, bool R12, bool DAG, int EPI, bool RED, int G>
 cudaError_t launch_shared_one(const HopArgs& a, cudaStream_t st) {
-    constexpr int G = kShGroups, NT = kShSites * G, S = kSharedStages;
+    constexpr int NT = kShSites * G, S = kSharedStages;
     constexpr int smem = shared_smem_bytes<P, R12, NT, S>();
     auto kern = wilson_hop_shared_kernel<P, R12, DAG, EPI, G, S, RED>;
     static bool configured = false;  // attribute set once per process (per instantiation)
@@ -327,30 +352,40 @@ cudaError_t launch_shared_one(const HopArgs& a, cudaStream_t st) {
     return launch_pdl(kern, dim3(tiles * a.nparity), dim3(NT), smem, st, a);
 }
 
-// Does a launch go to the shared-link kernel?  Several right-hand sides (or
-// slices) over whole parity blocks, at most 32 per group of threads.
-inline bool hop_shared_applies(const HopArgs& a) {
-    return a.nrhs >= 2 && a.nsite == 0 && a.site0 == 0 && a.nrhs <= 32 * kShGroups;
+// Does a launch go to the shared-link kernel?  Several right-hand sides (or slices) over whole
+// parity blocks, at most 32 per group of threads, and enough of them to repay the staging and
+// the barrier: on 16^2 x 24^2 the one-right-hand-side kernel takes 27.5 us for two FP32 ones (here
+// 30), 39.4 for three (36.5); with two-row FP16 links 51.6 us for five (53.6), 61.6 for six (58.7),
+// 119 for twelve (102).
+template <int P>
+bool hop_shared_applies(const HopArgs& a) {
+    return a.nrhs >= (P == LQ_F32 ? 3 : 6) && a.nsite == 0 && a.site0 == 0 && a.nrhs <= 32 * kShGroups;
 }
 
-template <int P>
-cudaError_t launch_hop_shared(const HopArgs& a, bool r12, bool dag, int epi, cudaStream_t st) {
+template <int P, bool R12, int G>
+cudaError_t launch_shared_groups(const HopArgs& a, bool dag, int epi, cudaStream_t st) {
     const bool red = a.red_partial != nullptr;
     if (red && epi == EPI_HOP) return cudaErrorInvalidValue;
-#define LQ_S_EPI(R, D)                                                                       \
-    switch (epi) {                                                                           \
-    case EPI_HOP: return launch_shared_one<P, R, D, EPI_HOP, false>(a, st);                  \
-    case EPI_DIAG: return red ? launch_shared_one<P, R, D, EPI_DIAG, true>(a, st)            \
-                              : launch_shared_one<P, R, D, EPI_DIAG, false>(a, st);          \
-    default: return red ? launch_shared_one<P, R, D, EPI_DWF, true>(a, st)                   \
-                        : launch_shared_one<P, R, D, EPI_DWF, false>(a, st);                 \
+#define LQ_S_EPI(D)                                                                               \
+    switch (epi) {                                                                                \
+    case EPI_HOP: return launch_shared_one<P, R12, D, EPI_HOP, false, G>(a, st);                  \
+    case EPI_DIAG: return red ? launch_shared_one<P, R12, D, EPI_DIAG, true, G>(a, st)            \
+                              : launch_shared_one<P, R12, D, EPI_DIAG, false, G>(a, st);          \
+    default: return red ? launch_shared_one<P, R12, D, EPI_DWF, true, G>(a, st)                   \
+                        : launch_shared_one<P, R12, D, EPI_DWF, false, G>(a, st);                 \
     }
-    if (r12) {
-        if (dag) { LQ_S_EPI(true, true) } else { LQ_S_EPI(true, false) }
-    } else {
-        if (dag) { LQ_S_EPI(false, true) } else { LQ_S_EPI(false, false) }
-    }
+    if (dag) { LQ_S_EPI(true) } else { LQ_S_EPI(false) }
 #undef LQ_S_EPI
+}
+
+template <int P, bool R12>
+cudaError_t launch_hop_shared(const HopArgs& a, bool dag, int epi, cudaStream_t st) {
+    // three groups instead of four where that leaves fewer idle in the last round; from twelve
+    // right-hand sides on four are as fast (FP32, same lattice: five 53.8 against 58.6 us, nine 84.5
+    // against 90.4, twelve 110.0 against 107.9)
+    const int n = a.nrhs;
+    if (n < 12 && 3 * ((n + 2) / 3) < 4 * ((n + 3) / 4)) return launch_shared_groups<P, R12, 3>(a, dag, epi, st);
+    return launch_shared_groups<P, R12, 4>(a, dag, epi, st);
 }
 
 }  // namespace lq
