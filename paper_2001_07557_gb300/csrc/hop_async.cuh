@@ -373,7 +373,7 @@ __device__ __forceinline__ void hop_async_site(const HopArgs& a, int i, int rhs,
             project_h2<P, MU, SG>(sw, hw);                                            \
             smem_words_link<P, NT>(stage, t, uw);                                     \
             su3_mul_h2<P, !FWD>(uw, hw, uh);                                          \
-            reconstruct_fma<MU, SG>(acc, uh, sgn ? -nrm : nrm);                       \
+            reconstruct_fma<MU, SG, true>(acc, uh, sgn ? -nrm : nrm);                 \
         } else if constexpr (NORM) {                                                  \
             smem_spinor<P, R12, NT>(stage, t, s, nrm);                                \
             project<MU, SG>(s, h);                                                    \

@@ -540,38 +540,53 @@ __device__ __forceinline__ void reconstruct_add(cplx<T> (&acc)[12], const cplx<T
     }
 }
 
+// d = a * b + d on two FP32 pairs, one instruction (the roundings of two scalar FMAs)
+__device__ __forceinline__ void fma2(cplx<float>& d, float a, cplx<float> b) {
+    asm("{\n\t.reg .b64 x, y, z;\n\t"
+        "mov.b64 x, {%2, %2};\n\tmov.b64 y, {%3, %4};\n\tmov.b64 z, {%0, %1};\n\t"
+        "fma.rn.f32x2 z, x, y, z;\n\tmov.b64 {%0, %1}, z;\n\t}"
+        : "+f"(d.re), "+f"(d.im)
+        : "f"(a), "f"(b.re), "f"(b.im));
+}
 // acc += n [uh; S A_mu^dag uh] with a run-time scale n (site norm x boundary phase):
 // every term is one FMA, so the scale costs nothing over reconstruct_add.
-template <typename T>
+template <bool PAIRS, typename T>
 __device__ __forceinline__ void cfma(cplx<T>& acc, T n, cplx<T> b) {
-    acc.re = fma(n, b.re, acc.re);
-    acc.im = fma(n, b.im, acc.im);
+    if constexpr (PAIRS) {
+        fma2(acc, n, b);
+    } else {
+        acc.re = fma(n, b.re, acc.re);
+        acc.im = fma(n, b.im, acc.im);
+    }
 }
 template <typename T>
 __device__ __forceinline__ void cfma_i(cplx<T>& acc, T n, cplx<T> b) {  // acc += n * i b
     acc.re = fma(-n, b.im, acc.re);
     acc.im = fma(n, b.re, acc.im);
 }
-template <int MU, int S, typename T>
+// PAIRS: (re, im) by one packed FP32 FMA, which helps the issue-bound kernel of hop_async.cuh
+// (24^3 x 48, 12 FP16 right-hand sides: 404 -> 394 us) and not the register-bound one of
+// hop_shared.cuh (416 -> 425).
+template <int MU, int S, bool PAIRS = false, typename T>
 __device__ __forceinline__ void reconstruct_fma(cplx<T> (&acc)[12], const cplx<T> (&uh)[6], T n) {
     const T sn = S > 0 ? n : -n;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const cplx<T> a = uh[c], b = uh[3 + c];
-        cfma(acc[c], n, a);
-        cfma(acc[3 + c], n, b);
+        cfma<PAIRS>(acc[c], n, a);
+        cfma<PAIRS>(acc[3 + c], n, b);
         if constexpr (MU == 0) {
             cfma_i(acc[6 + c], sn, b);
             cfma_i(acc[9 + c], sn, a);
         } else if constexpr (MU == 1) {
-            cfma(acc[6 + c], sn, b);
-            cfma(acc[9 + c], -sn, a);
+            cfma<PAIRS>(acc[6 + c], sn, b);
+            cfma<PAIRS>(acc[9 + c], -sn, a);
         } else if constexpr (MU == 2) {
             cfma_i(acc[6 + c], sn, a);
             cfma_i(acc[9 + c], -sn, b);
         } else {
-            cfma(acc[6 + c], sn, a);
-            cfma(acc[9 + c], sn, b);
+            cfma<PAIRS>(acc[6 + c], sn, a);
+            cfma<PAIRS>(acc[9 + c], sn, b);
         }
     }
 }
@@ -612,6 +627,23 @@ __device__ __forceinline__ uint32_t h2_adds(uint32_t a, uint32_t b) {
     else return h2_sub<P>(a, b);
 }
 
+// a + SG * i b: b's halves swapped, times (-SG, SG); the product is exact, so this rounds as an addition
+template <int P, int SG>
+__device__ __forceinline__ uint32_t h2_add_i(uint32_t a, uint32_t b) {
+    const uint32_t sw = __byte_perm(b, 0, 0x1032);
+    uint32_t k;
+    if constexpr (P == LQ_F16) {
+        k = SG > 0 ? 0x3c00bc00u : 0xbc003c00u;
+        __half2 r = __hfma2(*reinterpret_cast<const __half2*>(&sw), *reinterpret_cast<const __half2*>(&k),
+                            *reinterpret_cast<__half2*>(&a));
+        return *reinterpret_cast<uint32_t*>(&r);
+    } else {
+        k = SG > 0 ? 0x3f80bf80u : 0xbf803f80u;
+        __nv_bfloat162 r = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&sw),
+                                   *reinterpret_cast<const __nv_bfloat162*>(&k), *reinterpret_cast<__nv_bfloat162*>(&a));
+        return *reinterpret_cast<uint32_t*>(&r);
+    }
+}
 // (1 + S gamma_mu) psi projected on packed halves; same algebra as project()
 template <int P, int MU, int S>
 __device__ __forceinline__ void project_h2(const uint32_t (&s)[12], uint32_t (&h)[6]) {
@@ -619,14 +651,14 @@ __device__ __forceinline__ void project_h2(const uint32_t (&s)[12], uint32_t (&h
     for (int c = 0; c < 3; ++c) {
         const uint32_t p0 = s[c], p1 = s[3 + c], p2 = s[6 + c], p3 = s[9 + c];
         if constexpr (MU == 0) {
-            h[c] = h2_adds<P, -S>(p0, h2_mul_i(p3));
-            h[3 + c] = h2_adds<P, -S>(p1, h2_mul_i(p2));
+            h[c] = h2_add_i<P, -S>(p0, p3);
+            h[3 + c] = h2_add_i<P, -S>(p1, p2);
         } else if constexpr (MU == 1) {
             h[c] = h2_adds<P, -S>(p0, p3);
             h[3 + c] = h2_adds<P, S>(p1, p2);
         } else if constexpr (MU == 2) {
-            h[c] = h2_adds<P, -S>(p0, h2_mul_i(p2));
-            h[3 + c] = h2_adds<P, S>(p1, h2_mul_i(p3));
+            h[c] = h2_add_i<P, -S>(p0, p2);
+            h[3 + c] = h2_add_i<P, S>(p1, p3);
         } else {
             h[c] = h2_adds<P, S>(p0, p2);
             h[3 + c] = h2_adds<P, S>(p1, p3);
@@ -642,6 +674,19 @@ __device__ __forceinline__ float fma_h(unsigned short a, unsigned short b, float
     else asm("fma.rn.f32.bf16 %0, %1, %2, %3;" : "=f"(d) : "h"(a), "h"(b), "f"(c));
     return d;
 }
+// c - a b.  FP16: the negation folds into the instruction (24^3 x 48, 12 right-hand sides: 393 -> 369 us,
+// 32^4 step 144 -> 140); for BF16 it would cost one of its own, so nb, b with that part's sign
+// flipped beforehand, takes b's place.
+template <int P>
+__device__ __forceinline__ float fms_h(unsigned short a, unsigned short b, unsigned short nb, float c) {
+    if constexpr (P == LQ_F16) {
+        float d;
+        asm("{\n\t.reg .f16 t;\n\tneg.f16 t, %2;\n\tfma.rn.f32.f16 %0, %1, t, %3;\n\t}" : "=f"(d) : "h"(a), "h"(b), "f"(c));
+        return d;
+    } else {
+        return fma_h<P>(a, nb, c);
+    }
+}
 __device__ __forceinline__ unsigned short lo16(uint32_t w) { return (unsigned short)(w & 0xffffu); }
 __device__ __forceinline__ unsigned short hi16(uint32_t w) { return (unsigned short)(w >> 16); }
 
@@ -649,7 +694,7 @@ __device__ __forceinline__ unsigned short hi16(uint32_t w) { return (unsigned sh
 // FP16/BF16 and uh in FP32
 template <int P, bool ADJ>
 __device__ __forceinline__ void su3_mul_h2(const uint32_t (&u)[9], const uint32_t (&h)[6], cplx<float> (&uh)[6]) {
-    // copies of h with one part negated: -im (for U h) or -re (for U^dag h)
+    // copies of h with one part negated: -im (for U h) or -re (for U^dag h); used for BF16 only
     uint32_t hn[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) hn[k] = h[k] ^ (ADJ ? 0x00008000u : 0x80000000u);
@@ -665,7 +710,7 @@ __device__ __forceinline__ void su3_mul_h2(const uint32_t (&u)[9], const uint32_
                 if constexpr (!ADJ) {
                     // (a + ib)(c + id) = ac - bd + i(ad + bc)
                     re = fma_h<P>(lo16(w), lo16(x), re);
-                    re = fma_h<P>(hi16(w), hi16(xn), re);
+                    re = fms_h<P>(hi16(w), hi16(x), hi16(xn), re);
                     im = fma_h<P>(lo16(w), hi16(x), im);
                     im = fma_h<P>(hi16(w), lo16(x), im);
                 } else {
@@ -673,7 +718,7 @@ __device__ __forceinline__ void su3_mul_h2(const uint32_t (&u)[9], const uint32_
                     re = fma_h<P>(lo16(w), lo16(x), re);
                     re = fma_h<P>(hi16(w), hi16(x), re);
                     im = fma_h<P>(lo16(w), hi16(x), im);
-                    im = fma_h<P>(hi16(w), lo16(xn), im);
+                    im = fms_h<P>(hi16(w), lo16(x), lo16(xn), im);
                 }
             }
             uh[3 * sp + i] = {re, im};
