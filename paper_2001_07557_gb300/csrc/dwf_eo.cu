@@ -16,7 +16,11 @@
 // where z_end is z at the end of the sweep (s = Ls-1 forward, s = 0 backward).
 // A thread owns one (site, 16-byte plane) and sweeps twice over the Ls slices:
 // once for z_end, once to write y.  Each slice is read before it is written, so
-// the call may run in place.  O(Ls) work per component, bandwidth-bound.
+// the call may run in place.  O(Ls) work per component, bandwidth-bound, or, on
+// lattices that fit L2, bound by the latency of one slice after the other: both
+// kernels therefore load kBatch slices at a time (a load may not move above the
+// store of the slice before, as in and out may be one field).  12^3 x 24 x 11, FP32: the
+// combination 13.6 -> 7 us, the even-odd Moebius operator 77 -> 61 us (4, 6 or 8 alike).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -28,6 +32,8 @@
 namespace lq {
 
 namespace {
+
+constexpr int kBatch = 6;  // slices loaded before the first of them is used
 
 template <typename V, typename T>
 __device__ __forceinline__ V axpby4(T a, V x, T b, V y);  // a x + b y
@@ -68,10 +74,20 @@ __global__ void __launch_bounds__(256) m5inv_kernel(char* out, const char* in, i
     auto slice = [&](int j) { return fwd ? j : Ls - 1 - j; };
     V z = {};
     T w = g;
-    for (int j = 0; j < Ls; ++j) {
-        const V x = *reinterpret_cast<const V*>(src + (size_t)slice(j) * in_stride);
-        z = axpby4<V, T>(pc, x, g, z);
-        if (WITH_B && j + 1 < Ls) w *= g;
+    V x[kBatch];
+    auto load = [&](int j0) {
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b)
+            if (j0 + b < Ls) x[b] = *reinterpret_cast<const V*>(src + (size_t)slice(j0 + b) * in_stride);
+    };
+    for (int j0 = 0; j0 < Ls; j0 += kBatch) {
+        load(j0);
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            if (j0 + b >= Ls) break;
+            z = axpby4<V, T>(pc, x[b], g, z);
+            if (WITH_B && j0 + b + 1 < Ls) w *= g;
+        }
     }
     const V zend = z;
     V prev = {};
@@ -80,19 +96,23 @@ __global__ void __launch_bounds__(256) m5inv_kernel(char* out, const char* in, i
     T cw = -(T)mf_d * c5;  // S across the wall: -mf
     z = V{};
     w = g;
-    for (int j = 0; j < Ls; ++j) {
-        const int s = slice(j);
-        const V x = *reinterpret_cast<const V*>(src + (size_t)s * in_stride);
-        z = axpby4<V, T>(pc, x, g, z);
-        const V y = axpby4<V, T>((T)1, z, -c * w, zend);
-        if constexpr (WITH_B) {
-            *reinterpret_cast<V*>(dst + (size_t)s * out_stride) = axpby4<V, T>(b5, y, cw, prev);
-            prev = y;
-            cw = c5;
-        } else {
-            *reinterpret_cast<V*>(dst + (size_t)s * out_stride) = y;
+    for (int j0 = 0; j0 < Ls; j0 += kBatch) {
+        if (j0 > 0 || Ls > kBatch) load(j0);  // (else the first sweep's loads are still here)
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            if (j0 + b >= Ls) break;
+            const int s = slice(j0 + b);
+            z = axpby4<V, T>(pc, x[b], g, z);
+            const V y = axpby4<V, T>((T)1, z, -c * w, zend);
+            if constexpr (WITH_B) {
+                *reinterpret_cast<V*>(dst + (size_t)s * out_stride) = axpby4<V, T>(b5, y, cw, prev);
+                prev = y;
+                cw = c5;
+            } else {
+                *reinterpret_cast<V*>(dst + (size_t)s * out_stride) = y;
+            }
+            w *= g;
         }
-        w *= g;
     }
 }
 
@@ -100,9 +120,11 @@ __global__ void __launch_bounds__(256) m5inv_kernel(char* out, const char* in, i
 // with S psi(s) = P- psi(s+1) + P+ psi(s-1), walls -mf.  For planes of spins 0,1
 // (P+) S reads slice s-1, for spins 2,3 (P-) slice s+1; the dagger swaps them.
 // Fields: Ls slices at slice_stride bytes, each nblk parity blocks of Vh sites.
-// One thread per (block, plane, site) walks the slices.
+// One thread per (block, plane, site) walks the slices in the order in which S reads the
+// one before, so that each is read once.
 template <int P>
-__global__ void __launch_bounds__(256) m5_lincomb_kernel(char* out, const char* u, const char* v, int Vh, int nblk,
+__global__ void __launch_bounds__(256) m5_lincomb_kernel(char* __restrict__ out, const char* __restrict__ u,
+                                                         const char* __restrict__ v, int Vh, int nblk,
                                                          size_t slice_stride, int Ls, double a_d, double b_d,
                                                          double c_d, double d_d, double mf_d, int dag) {
     pdl_enter();
@@ -117,15 +139,30 @@ __global__ void __launch_bounds__(256) m5_lincomb_kernel(char* out, const char* 
     const bool down = (k < NPL / 2) != (dag != 0);  // S reads slice s-1 (else s+1)
     const size_t off = (size_t)blk * NPL * Vh * sizeof(V) + ((size_t)k * Vh + i) * sizeof(V);
     const T a = (T)a_d, b = (T)b_d, c = (T)c_d, d = (T)d_d, mf = (T)mf_d;
-    auto at = [&](const char* f, int s) { return *reinterpret_cast<const V*>(f + (size_t)s * slice_stride + off); };
-    for (int s = 0; s < Ls; ++s) {
-        int sn = down ? s - 1 : s + 1;
-        T w = 1;
-        if (sn < 0) sn = Ls - 1, w = -mf;
-        if (sn >= Ls) sn = 0, w = -mf;
-        V r = axpby4<V, T>(a, at(u, s), b * w, at(u, sn));
-        if (v) r = axpby4<V, T>((T)1, r, (T)1, axpby4<V, T>(c, at(v, s), d * w, at(v, sn)));
-        *reinterpret_cast<V*>(out + (size_t)s * slice_stride + off) = r;
+    auto slice = [&](int j) { return (size_t)(down ? j : Ls - 1 - j) * slice_stride + off; };
+    auto at = [&](const char* f, int j) { return *reinterpret_cast<const V*>(f + slice(j)); };
+    V up = at(u, Ls - 1), vp = {};  // what S reads for the first slice: the last one, times -mf
+    if (v) vp = at(v, Ls - 1);
+    T w = -mf;
+    for (int j0 = 0; j0 < Ls; j0 += kBatch) {
+        V us[kBatch], vs[kBatch];
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q) {
+            if (j0 + q < Ls) us[q] = at(u, j0 + q);
+            if (v && j0 + q < Ls) vs[q] = at(v, j0 + q);
+        }
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q) {
+            if (j0 + q >= Ls) break;
+            V r = axpby4<V, T>(a, us[q], b * w, up);
+            up = us[q];
+            if (v) {
+                r = axpby4<V, T>((T)1, r, (T)1, axpby4<V, T>(c, vs[q], d * w, vp));
+                vp = vs[q];
+            }
+            *reinterpret_cast<V*>(out + slice(j0 + q)) = r;
+            w = 1;
+        }
     }
 }
 
