@@ -22,18 +22,28 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Block-reduce v; thread 0 writes the partial, and the last block of this rhs
-// returns true in every thread with `total` set (fixed-order sum of partials).
-__device__ bool reduce_last(double v, double* partial, unsigned* ticket, int nblk_x, double& total) {
-    __shared__ double ws[kThreads / 32];
-    __shared__ bool last;
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) ws[wid] = v;
+// Sum v over the block; valid in thread 0.  An addition of a warp occupies the FP64 unit for 77 clocks
+// whatever its lanes hold, so one warp adds up all threads' values (13 additions a block) instead
+// of every warp its own (40 and 8).
+__device__ __forceinline__ double block_sum(double v, double* ws) {
+    ws[threadIdx.x] = v;
     __syncthreads();
+    double s = 0;
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) s += ws[w * 32 + threadIdx.x];
+        s = warp_sum(s);
+    }
+    return s;
+}
+
+// Block-reduce v; thread 0 writes the partial, and the last block of this rhs
+// returns true in every thread with `total` set in thread 0 (fixed-order sum of partials).
+__device__ bool reduce_last(double v, double* partial, unsigned* ticket, int nblk_x, double& total) {
+    __shared__ double ws[kThreads];
+    __shared__ bool last;
+    const double s = block_sum(v, ws);
     if (threadIdx.x == 0) {
-        double s = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += ws[w];
         partial[blockIdx.x] = s;
         __threadfence();
         const unsigned t = atomicAdd(ticket, 1u);
@@ -42,20 +52,14 @@ __device__ bool reduce_last(double v, double* partial, unsigned* ticket, int nbl
     __syncthreads();
     if (!last) return false;
     __threadfence();
-    double s = 0;
-    for (int b = threadIdx.x; b < nblk_x; b += blockDim.x) s += __ldcg(partial + b);
+    double t = 0;
+    for (int b = threadIdx.x; b < nblk_x; b += blockDim.x) t += __ldcg(partial + b);
     // deterministic: fixed thread -> partial assignment, then a fixed-shape tree
-    s = warp_sum(s);
-    __syncthreads();
-    if (lane == 0) ws[wid] = s;
-    __syncthreads();
+    t = block_sum(t, ws);
     if (threadIdx.x == 0) {
-        double t = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += ws[w];
         total = t;
         *ticket = 0;  // ready for the next launch
     }
-    __syncthreads();
     return true;
 }
 
@@ -95,7 +99,7 @@ __global__ void __launch_bounds__(kThreads) dot_kernel(VecRef a, VecRef b, int V
         T site = 0;
 #pragma unroll
         for (int k = 0; k < 12; ++k) site += sa[k].re * sb[k].re + sa[k].im * sb[k].im;
-        acc += (double)site;
+        acc += widen(site);
     }
     double total;
     if (!reduce_last(acc, scratch + (size_t)rhs * gridDim.x, tickets + rhs, gridDim.x, total)) return;
@@ -115,41 +119,50 @@ __global__ void __launch_bounds__(kThreads) dot_kernel(VecRef a, VecRef b, int V
     }
 }
 
-// x += alpha p ; r -= alpha q ; rr_new = |r|^2 ; beta, convergence (per rhs)
-template <int PX, int PP, int PR, int PQ>
-__global__ void __launch_bounds__(kThreads) cg_update_kernel(VecRef x, VecRef p, VecRef r, VecRef q, int Vh, int nblk,
-                                                             double* scratch, unsigned* tickets, CgScalars* st) {
+// The vector part of two CG steps, even and odd, with search directions p0 and p1:
+//   even: r -= alpha q;  p1 = r + beta p0
+//   odd:  r -= alpha q;  x += alpha_even p0 + alpha_odd p1;  p0 = r + beta p1
+// x is read and written every other step: FP32 x with FP16 r, p, q move 434 bytes a site and step
+// instead of 556 (HBM-bound; with the shorter reductions below, 12-source batched CG on 24^3 x 48
+// 195.5 -> 190.0 ms, mixed CG on 32^4 33.6 -> 33.0 ms).  The additions to x are those of a step at a time, in the same order.
+// pend holds the alphas whose alpha p is not in x yet; a right-hand side that finishes in the even
+// step leaves pend = {alpha, 0} to the odd one, and the next pair's even step clears it.
+
+// r -= alpha q ; rr_new = |r|^2 ; beta, convergence (per rhs)
+template <int PR, int PQ>
+__global__ void __launch_bounds__(kThreads) cg_r_update_kernel(VecRef r, VecRef q, int Vh, int nblk, double* scratch,
+                                                               unsigned* tickets, CgScalars* st, int odd) {
     pdl_enter();
     const int rhs = blockIdx.y;
     CgScalars& s = st[rhs];
-    if (s.done) return;
-    using T = Compute<PX, PP, PR, PQ>;
+    if (s.done) {
+        if (!odd && blockIdx.x == 0 && threadIdx.x == 0) s.pend[0] = s.pend[1] = 0;
+        return;
+    }
+    using T = Compute<PR, PQ>;
     const T alpha = (T)s.alpha;
     double acc = 0;
     const long n = (long)Vh * nblk;
     for (long j = (long)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (long)gridDim.x * blockDim.x) {
         const int bk = (int)(j / Vh), i = (int)(j - (long)bk * Vh);
-        cplx<T> xs[12], ps[12], rs[12], qs[12];
-        load_spinor<PX, T>(blk_ptr<PX, T>(x, rhs, bk, Vh), Vh, i, xs);
-        load_spinor<PP, T>(blk_ptr<PP, T>(p, rhs, bk, Vh), Vh, i, ps);
+        cplx<T> rs[12], qs[12];
         load_spinor<PR, T>(blk_ptr<PR, T>(r, rhs, bk, Vh), Vh, i, rs);
         load_spinor<PQ, T>(blk_ptr<PQ, T>(q, rhs, bk, Vh), Vh, i, qs);
         T site = 0;
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            xs[k].re = fma(alpha, ps[k].re, xs[k].re);
-            xs[k].im = fma(alpha, ps[k].im, xs[k].im);
             rs[k].re = fma(-alpha, qs[k].re, rs[k].re);
             rs[k].im = fma(-alpha, qs[k].im, rs[k].im);
             site += rs[k].re * rs[k].re + rs[k].im * rs[k].im;
         }
-        acc += (double)site;
-        store_spinor<PX, T>(const_cast<char*>(blk_ptr<PX, T>(x, rhs, bk, Vh)), Vh, i, xs);
+        acc += widen(site);
         store_spinor<PR, T>(const_cast<char*>(blk_ptr<PR, T>(r, rhs, bk, Vh)), Vh, i, rs);
     }
     double total;
     if (!reduce_last(acc, scratch + (size_t)rhs * gridDim.x, tickets + rhs, gridDim.x, total)) return;
     if (threadIdx.x != 0) return;
+    s.pend[odd] = s.alpha;
+    if (!odd) s.pend[1] = 0;
     s.iter += 1;
     if (!finite(total)) {
         s.done = 1;
@@ -165,9 +178,10 @@ __global__ void __launch_bounds__(kThreads) cg_update_kernel(VecRef x, VecRef p,
     }
 }
 
-// p = r + beta p
+// pn = r + beta p
 template <int PP, int PR>
-__global__ void __launch_bounds__(kThreads) cg_xpay_kernel(VecRef p, VecRef r, int Vh, int nblk, const CgScalars* st) {
+__global__ void __launch_bounds__(kThreads) cg_xpay_kernel(VecRef pn, VecRef p, VecRef r, int Vh, int nblk,
+                                                           const CgScalars* st) {
     pdl_enter();
     const int rhs = blockIdx.y;
     if (st[rhs].done) return;
@@ -184,7 +198,54 @@ __global__ void __launch_bounds__(kThreads) cg_xpay_kernel(VecRef p, VecRef r, i
             ps[k].re = fma(beta, ps[k].re, rs[k].re);
             ps[k].im = fma(beta, ps[k].im, rs[k].im);
         }
-        store_spinor<PP, T>(const_cast<char*>(blk_ptr<PP, T>(p, rhs, bk, Vh)), Vh, i, ps);
+        store_spinor<PP, T>(const_cast<char*>(blk_ptr<PP, T>(pn, rhs, bk, Vh)), Vh, i, ps);
+    }
+}
+
+// x += pend[0] p0 + pend[1] p1 ; p0 = r + beta p1 unless the right-hand side is done
+template <int PX, int PP, int PR>
+__global__ void __launch_bounds__(kThreads) cg_x_xpay_kernel(VecRef x, VecRef p0, VecRef p1, VecRef r, int Vh,
+                                                             int nblk, const CgScalars* st) {
+    pdl_enter();
+    const int rhs = blockIdx.y;
+    const CgScalars& s = st[rhs];
+    const bool go = !s.done, two = s.pend[1] != 0;
+    if (!go && s.pend[0] == 0 && !two) return;
+    using TX = Compute<PX, PP>;
+    using T = Compute<PP, PR>;
+    const TX a0 = (TX)s.pend[0], a1 = (TX)s.pend[1];
+    const T beta = (T)s.beta;
+    const long n = (long)Vh * nblk;
+    for (long j = (long)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (long)gridDim.x * blockDim.x) {
+        const int bk = (int)(j / Vh), i = (int)(j - (long)bk * Vh);
+        cplx<TX> xs[12], ps[12];
+        cplx<T> qs[12];
+        load_spinor<PX, TX>(blk_ptr<PX, TX>(x, rhs, bk, Vh), Vh, i, xs);
+        load_spinor<PP, TX>(blk_ptr<PP, TX>(p0, rhs, bk, Vh), Vh, i, ps);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            xs[k].re = fma(a0, ps[k].re, xs[k].re);
+            xs[k].im = fma(a0, ps[k].im, xs[k].im);
+        }
+        if (go || two) {  // (p1 may be unset where the even step was the last)
+            load_spinor<PP, T>(blk_ptr<PP, T>(p1, rhs, bk, Vh), Vh, i, qs);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {
+                xs[k].re = fma(a1, (TX)qs[k].re, xs[k].re);
+                xs[k].im = fma(a1, (TX)qs[k].im, xs[k].im);
+            }
+        }
+        store_spinor<PX, TX>(const_cast<char*>(blk_ptr<PX, TX>(x, rhs, bk, Vh)), Vh, i, xs);
+        if (go) {
+            cplx<T> rs[12];
+            load_spinor<PR, T>(blk_ptr<PR, T>(r, rhs, bk, Vh), Vh, i, rs);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {
+                qs[k].re = fma(beta, qs[k].re, rs[k].re);
+                qs[k].im = fma(beta, qs[k].im, rs[k].im);
+            }
+            store_spinor<PP, T>(const_cast<char*>(blk_ptr<PP, T>(p0, rhs, bk, Vh)), Vh, i, qs);
+        }
     }
 }
 
@@ -231,6 +292,7 @@ __global__ void cg_init_kernel(CgScalars* st, const double* rr, const double* bb
     s.maxiter = maxiter;
     s.status = LQ_OK;
     s.alpha = s.beta = s.pAp = 0;
+    s.pend[0] = s.pend[1] = 0;
     s.done = (rr[k] <= s.stop2) ? 1 : 0;
     if (!isfinite(rr[k])) {
         s.done = 1;
@@ -313,7 +375,7 @@ __device__ __forceinline__ void load_site(const char* base, size_t rhs_stride, i
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
             float2 v = q[k];
-            s[k] = {(double)v.x, (double)v.y};
+            s[k] = {widen(v.x), widen(v.y)};
         }
     }
 }
@@ -408,7 +470,7 @@ __global__ void __launch_bounds__(kThreads) bdot_alpha_kernel(const BSeg* __rest
         T site = 0;
 #pragma unroll
         for (int k = 0; k < 12; ++k) site += a[k].re * b[k].re + a[k].im * b[k].im;
-        acc += (double)site;
+        acc += widen(site);
     }
     double total;
     if (!reduce_last(acc, sg.partial, sg.ticket, gridDim.x, total)) return;
@@ -450,7 +512,7 @@ __global__ void __launch_bounds__(kThreads) bupdate_kernel(const BSeg* __restric
             rs[k].im = fma(-alpha, qs[k].im, rs[k].im);
             site += rs[k].re * rs[k].re + rs[k].im * rs[k].im;
         }
-        acc += (double)site;
+        acc += widen(site);
         store_spinor<PX, T>(const_cast<char*>(seg_blk<PX>(sg.x, bk, sg.Vh)), sg.Vh, i, xs);
         store_spinor<PX, T>(const_cast<char*>(seg_blk<PX>(sg.r, bk, sg.Vh)), sg.Vh, i, rs);
     }
@@ -562,35 +624,39 @@ cudaError_t launch_dot(const VecRef& a, const VecRef& b, int Vh, int nblk, int n
     return cudaGetLastError();
 }
 
-cudaError_t launch_cg_update(const VecRef& x, const VecRef& p, const VecRef& r, const VecRef& q, int Vh, int nblk,
-                             int nrhs, const Scratch& sc, CgScalars* st, cudaStream_t s) {
+// precision combinations used by the solvers: all equal (FP64 or FP32); x in FP32 with r, p, q in
+// FP16 or BF16
+cudaError_t launch_cg_r_update(const VecRef& r, const VecRef& q, int Vh, int nblk, int nrhs, const Scratch& sc,
+                               CgScalars* st, int odd, cudaStream_t s) {
     dim3 grid(grid_x(Vh, nblk), nrhs);
-    // precision combinations used by the solvers: all equal; x, r in FP32 with p, q in FP16/BF16;
-    // x in FP32 with r, p, q in FP16/BF16
-    if (x.prec == LQ_F64 && p.prec == LQ_F64 && r.prec == LQ_F64 && q.prec == LQ_F64)
-        launch_pdl(cg_update_kernel<LQ_F64, LQ_F64, LQ_F64, LQ_F64>, grid, kThreads, 0, s, x, p, r, q, Vh, nblk, sc.partial, sc.tickets, st);
-    else if (x.prec == LQ_F32 && r.prec == LQ_F32 && p.prec == q.prec) {
-        switch (p.prec) {
-        case LQ_F32: launch_pdl(cg_update_kernel<LQ_F32, LQ_F32, LQ_F32, LQ_F32>, grid, kThreads, 0, s, x, p, r, q, Vh, nblk, sc.partial, sc.tickets, st); break;
-        case LQ_F16: launch_pdl(cg_update_kernel<LQ_F32, LQ_F16, LQ_F32, LQ_F16>, grid, kThreads, 0, s, x, p, r, q, Vh, nblk, sc.partial, sc.tickets, st); break;
-        case LQ_BF16: launch_pdl(cg_update_kernel<LQ_F32, LQ_BF16, LQ_F32, LQ_BF16>, grid, kThreads, 0, s, x, p, r, q, Vh, nblk, sc.partial, sc.tickets, st); break;
-        default: return cudaErrorInvalidValue;
-        }
-    } else if (x.prec == LQ_F32 && r.prec == p.prec && p.prec == q.prec && p.prec == LQ_F16) {
-        launch_pdl(cg_update_kernel<LQ_F32, LQ_F16, LQ_F16, LQ_F16>, grid, kThreads, 0, s, x, p, r, q, Vh, nblk, sc.partial, sc.tickets, st);
-    } else if (x.prec == LQ_F32 && r.prec == p.prec && p.prec == q.prec && p.prec == LQ_BF16) {
-        launch_pdl(cg_update_kernel<LQ_F32, LQ_BF16, LQ_BF16, LQ_BF16>, grid, kThreads, 0, s, x, p, r, q, Vh, nblk, sc.partial, sc.tickets, st);
-    } else {
-        return cudaErrorInvalidValue;
-    }
+    if (r.prec != q.prec) return cudaErrorInvalidValue;
+    LQ_P_SWITCH(r.prec, P, (launch_pdl(cg_r_update_kernel<P, P>, grid, kThreads, 0, s, r, q, Vh, nblk, sc.partial, sc.tickets, st, odd)))
     return cudaGetLastError();
 }
 
-cudaError_t launch_cg_xpay(const VecRef& p, const VecRef& r, int Vh, int nblk, int nrhs, const CgScalars* st,
-                           cudaStream_t s) {
+cudaError_t launch_cg_xpay(const VecRef& pn, const VecRef& p, const VecRef& r, int Vh, int nblk, int nrhs,
+                           const CgScalars* st, cudaStream_t s) {
     dim3 grid(grid_x(Vh, nblk), nrhs);
-    LQ_P_SWITCH(p.prec, PP, LQ_P_SWITCH(r.prec, PR,
-        (launch_pdl(cg_xpay_kernel<PP, PR>, grid, kThreads, 0, s, p, r, Vh, nblk, st))))
+    if (r.prec != p.prec || pn.prec != p.prec) return cudaErrorInvalidValue;
+    LQ_P_SWITCH(p.prec, P, (launch_pdl(cg_xpay_kernel<P, P>, grid, kThreads, 0, s, pn, p, r, Vh, nblk, st)))
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cg_x_xpay(const VecRef& x, const VecRef& p0, const VecRef& p1, const VecRef& r, int Vh, int nblk,
+                             int nrhs, const CgScalars* st, cudaStream_t s) {
+    dim3 grid(grid_x(Vh, nblk), nrhs);
+    if (r.prec != p0.prec || p1.prec != p0.prec) return cudaErrorInvalidValue;
+    if (x.prec == LQ_F64 && p0.prec == LQ_F64) {
+        launch_pdl(cg_x_xpay_kernel<LQ_F64, LQ_F64, LQ_F64>, grid, kThreads, 0, s, x, p0, p1, r, Vh, nblk, st);
+        return cudaGetLastError();
+    }
+    if (x.prec != LQ_F32) return cudaErrorInvalidValue;
+    switch (p0.prec) {
+    case LQ_F32: launch_pdl(cg_x_xpay_kernel<LQ_F32, LQ_F32, LQ_F32>, grid, kThreads, 0, s, x, p0, p1, r, Vh, nblk, st); break;
+    case LQ_F16: launch_pdl(cg_x_xpay_kernel<LQ_F32, LQ_F16, LQ_F16>, grid, kThreads, 0, s, x, p0, p1, r, Vh, nblk, st); break;
+    case LQ_BF16: launch_pdl(cg_x_xpay_kernel<LQ_F32, LQ_BF16, LQ_BF16>, grid, kThreads, 0, s, x, p0, p1, r, Vh, nblk, st); break;
+    default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 

@@ -49,10 +49,14 @@ cudaError_t launch_bxpay(const BSeg* segs, int nseg, int gx, int pp, int pr, cud
 
 cudaError_t launch_dot(const VecRef& a, const VecRef& b, int Vh, int nblk, int nrhs, const Scratch& sc,
                        CgScalars* st, double* out, int fin, cudaStream_t s);
-cudaError_t launch_cg_update(const VecRef& x, const VecRef& p, const VecRef& r, const VecRef& q, int Vh, int nblk,
-                             int nrhs, const Scratch& sc, CgScalars* st, cudaStream_t s);
-cudaError_t launch_cg_xpay(const VecRef& p, const VecRef& r, int Vh, int nblk, int nrhs, const CgScalars* st,
-                           cudaStream_t s);
+// The vector part of a pair of CG steps (odd = 0, then 1), with search directions p0 and p1 in turn:
+// launch_cg_r_update(odd 0), launch_cg_xpay(p1, p0, r); launch_cg_r_update(odd 1), launch_cg_x_xpay.
+cudaError_t launch_cg_r_update(const VecRef& r, const VecRef& q, int Vh, int nblk, int nrhs, const Scratch& sc,
+                               CgScalars* st, int odd, cudaStream_t s);
+cudaError_t launch_cg_xpay(const VecRef& pn, const VecRef& p, const VecRef& r, int Vh, int nblk, int nrhs,
+                           const CgScalars* st, cudaStream_t s);
+cudaError_t launch_cg_x_xpay(const VecRef& x, const VecRef& p0, const VecRef& p1, const VecRef& r, int Vh, int nblk,
+                             int nrhs, const CgScalars* st, cudaStream_t s);
 cudaError_t launch_axpby(const VecRef& y, const VecRef& x, double a, double b, int Vh, int nblk, int nrhs,
                          cudaStream_t s);
 // Sum the warp partials of the last fused-norm hop (ngroups groups of nwarps

@@ -28,7 +28,7 @@ namespace lq {
 
 namespace {
 
-constexpr int kItersPerGraph = 8;
+constexpr int kItersPerGraph = 8;  // even: whole pairs of steps
 
 struct OpGeom {
     int op;
@@ -198,6 +198,9 @@ int run_cg(lq_handle* h, const OpGeom& og, const Ctl& c, int pp, const VecRef& e
     CgVecs v;
     int rc = cg_vectors(h, og, pr, pp, slot0, &v);
     if (rc) return rc;
+    void* pbuf;  // the second search direction
+    if ((rc = ensure_ws(h, WS_CGP, og.bytes(h, pp), &pbuf))) return rc;
+    const VecRef p2[2] = {v.p, og.ref(h, pbuf, pp)};
     const char* L;
     size_t lb;
     if ((rc = get_links(h, pp, &L, &lb, s))) return rc;  // pack before any capture
@@ -220,7 +223,8 @@ int run_cg(lq_handle* h, const OpGeom& og, const Ctl& c, int pp, const VecRef& e
         return LQ_ERR_CUDA;
     if (launch_cg_init(c.st, c.red, c.red, tol, maxiter, og.nrhs, s) != cudaSuccess) return LQ_ERR_CUDA;
 
-    // one graph = kItersPerGraph iterations; finished right-hand sides skip every launch
+    // one graph = kItersPerGraph iterations (pairs of steps, x updated in the second); finished
+    // right-hand sides skip every launch
     h->skip = &c.st[0].done;
     h->skip_stride = (int)(sizeof(CgScalars) / sizeof(int));
     cudaGraph_t graph = nullptr;
@@ -229,15 +233,17 @@ int run_cg(lq_handle* h, const OpGeom& og, const Ctl& c, int pp, const VecRef& e
     if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) rc = LQ_ERR_CUDA;
     for (int k = 0; k < kItersPerGraph && rc == LQ_OK; ++k) {
         // q = K^dag K p, with <p, q> = |K p|^2 and alpha fused into the launch that writes K p
-        rc = apply_normal(h, og, pp, v.q.ptr, v.p.ptr, v.t.ptr, v.tmp.ptr, s, &c);
+        const int odd = k & 1;
+        rc = apply_normal(h, og, pp, v.q.ptr, p2[odd].ptr, v.t.ptr, v.tmp.ptr, s, &c);
         if (rc) break;
         if (launch_hop_norm_finalize(c.hop_partial, hop_warps(h, og), og.op == LQ_OP_DWF_NORMAL ? 1 : og.nrhs, c.st,
                                      c.sc, Vh, og.nblk, s) != cudaSuccess) {
             rc = LQ_ERR_CUDA;
             break;
         }
-        if (launch_cg_update(e, v.p, v.r, v.q, Vh, og.nblk, og.nrhs, c.sc, c.st, s) != cudaSuccess ||
-            launch_cg_xpay(v.p, v.r, Vh, og.nblk, og.nrhs, c.st, s) != cudaSuccess)
+        if (launch_cg_r_update(v.r, v.q, Vh, og.nblk, og.nrhs, c.sc, c.st, odd, s) != cudaSuccess ||
+            (odd ? launch_cg_x_xpay(e, p2[0], p2[1], v.r, Vh, og.nblk, og.nrhs, c.st, s)
+                 : launch_cg_xpay(p2[1], p2[0], v.r, Vh, og.nblk, og.nrhs, c.st, s)) != cudaSuccess)
             rc = LQ_ERR_CUDA;
     }
     cudaError_t ce = cudaStreamEndCapture(s, &graph);

@@ -52,7 +52,7 @@ __device__ __forceinline__ void hop_norm_site(const HopArgs& a, const cplx<T> (&
     double v = 0;
     if (active) {
 #pragma unroll
-        for (int k = 0; k < 12; ++k) v += (double)(o[k].re * o[k].re + o[k].im * o[k].im);
+        for (int k = 0; k < 12; ++k) v += widen(o[k].re * o[k].re + o[k].im * o[k].im);
     }
     const int wpb = blockDim.x >> 5;
     const int grp = EPI == EPI_DWF ? 0 : rhs;

@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(NT) wilson_hop_async_kernel(const HopArgs a) {
             T q = 0;
 #pragma unroll
             for (int k = 0; k < 12; ++k) q += o[k].re * o[k].re + o[k].im * o[k].im;
-            v = (double)q;
+            v = widen(q);
         }
         // warp partials, group-major: [group][warp of the group's blocks]
         const int wpb = blockDim.x >> 5;

@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(kShSites* G, shared_min_blocks<P, G>()) wilson
                 T q = 0;
 #pragma unroll
                 for (int k = 0; k < 12; ++k) q += o[k].re * o[k].re + o[k].im * o[k].im;
-                v = (double)q;
+                v = widen(q);
             }
             const int dwf = EPI == EPI_DWF;
             hop_norm_warp(v, a.red_partial, (int)shared_red_slot(a, dwf, rhs, pidx, tile * (NS / 32) + (s >> 5)));

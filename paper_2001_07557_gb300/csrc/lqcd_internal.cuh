@@ -61,6 +61,7 @@ struct CgScalars {
     double pAp;
     double alpha;
     double beta;
+    double pend[2];  // alphas of the even and the odd step of a pair whose alpha p is not in x yet (cg_r_update)
     int iter;
     int maxiter;
     int done;      // converged, broke down, or out of iterations
@@ -215,8 +216,13 @@ __device__ __forceinline__ void load_spinor(const char* __restrict__ blk, int Vh
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             float4 v = __ldg(q + (size_t)k * Vh + i);
-            s[2 * k] = {(T)v.x, (T)v.y};
-            s[2 * k + 1] = {(T)v.z, (T)v.w};
+            if constexpr (sizeof(T) == 8) {
+                s[2 * k] = {widen(v.x), widen(v.y)};
+                s[2 * k + 1] = {widen(v.z), widen(v.w)};
+            } else {
+                s[2 * k] = {(T)v.x, (T)v.y};
+                s[2 * k + 1] = {(T)v.z, (T)v.w};
+            }
         }
     } else {
         const uint4* q = reinterpret_cast<const uint4*>(blk);
@@ -226,10 +232,14 @@ __device__ __forceinline__ void load_spinor(const char* __restrict__ blk, int Vh
         for (int k = 0; k < 3; ++k) {
             uint4 v = __ldg(q + (size_t)k * Vh + i);
             float2 a = h2f(v.x, tag), b = h2f(v.y, tag), c = h2f(v.z, tag), d = h2f(v.w, tag);
-            s[4 * k + 0] = {a.x * nrm, a.y * nrm};
-            s[4 * k + 1] = {b.x * nrm, b.y * nrm};
-            s[4 * k + 2] = {c.x * nrm, c.y * nrm};
-            s[4 * k + 3] = {d.x * nrm, d.y * nrm};
+            auto put = [&](int j, float2 w) {
+                if constexpr (sizeof(T) == 8) s[4 * k + j] = {widen(w.x * nrm), widen(w.y * nrm)};
+                else s[4 * k + j] = {(T)(w.x * nrm), (T)(w.y * nrm)};
+            };
+            put(0, a);
+            put(1, b);
+            put(2, c);
+            put(3, d);
         }
     }
 }
