@@ -8,6 +8,7 @@
 #include <cstring>
 
 #include "lqcd_kernels.h"
+#include "pdl.cuh"
 
 namespace lq {
 
@@ -51,6 +52,7 @@ using ConvT = typename std::conditional<DP == LQ_F64 || SP == LQ_F64, double, fl
 template <int DP, int SP>
 __global__ void __launch_bounds__(kBlock) spinor_to_native_kernel(char* nat, const void* sm, Geom g, bool full,
                                                                   int parity, int nparity) {
+    pdl_enter();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.Vh) return;
     const int pi = blockIdx.y % nparity;
@@ -76,6 +78,9 @@ __global__ void __launch_bounds__(kBlock) spinor_from_native_kernel(void* sm, co
     constexpr int PITCH = CH + 1;
     __shared__ uint4 slots[kBlock * PITCH];
     __shared__ size_t where[kBlock];
+    // No early start of the next launch (pdl_enter): a spinor_to_native_kernel that follows would find
+    // L1 cut to what this kernel's shared memory leaves (16^4, FP64: 53.2 against 50.1 us).
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int t = threadIdx.x, w = t & ~31, lane = t & 31;
     const int i = blockIdx.x * kBlock + t;
     const int pi = blockIdx.y % nparity;
@@ -250,30 +255,44 @@ __global__ void link_fixed_check_kernel(const T* src, long nlinks, unsigned* bad
     default: { constexpr int DP = LQ_BF16; BODY; } break;    \
     }
 
+// A conversion to or from site-major of up to four blocks per SM is launched as a programmatic
+// dependent: what it takes there is the launch (D on FP64 site-major fields, 4^4: 20.6 -> 16.0 us,
+// 8^3 x 16: 20.9 -> 17.8, 16^4: 51.6 -> 50.1).  A larger one is not: started beside the end of a hop,
+// which holds most of L1 as shared memory, spinor_to_native_kernel lacks the L1 that gathers its 16-byte
+// reads into lines (32^4 FP64 after an FP32 hop: 163 -> 227 us for the two).
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_conversion(void (*kern)(KArgs...), dim3 grid, cudaStream_t st, Args... args) {
+    if (grid.x * (size_t)grid.y <= 4 * 152) return launch_pdl(kern, grid, dim3(kBlock), 0, st, args...);
+    kern<<<grid, kBlock, 0, st>>>(args...);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_spinor_to_native(int dst_prec, void* dst, int src_prec, const void* src, const Geom& g, bool full,
                                     int parity, int nrhs, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
     const int np = full ? 2 : 1;
     dim3 grid((g.Vh + kBlock - 1) / kBlock, nrhs * np);
     char* d = static_cast<char*>(dst);
     if (src_prec == LQ_F64) {
-        LQ_DP_SWITCH(dst_prec, (spinor_to_native_kernel<DP, LQ_F64><<<grid, kBlock, 0, st>>>(d, src, g, full, parity, np)))
+        LQ_DP_SWITCH(dst_prec, e = launch_conversion(spinor_to_native_kernel<DP, LQ_F64>, grid, st, d, src, g, full, parity, np))
     } else {
-        LQ_DP_SWITCH(dst_prec, (spinor_to_native_kernel<DP, LQ_F32><<<grid, kBlock, 0, st>>>(d, src, g, full, parity, np)))
+        LQ_DP_SWITCH(dst_prec, e = launch_conversion(spinor_to_native_kernel<DP, LQ_F32>, grid, st, d, src, g, full, parity, np))
     }
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_spinor_from_native(int dst_prec, void* dst, int src_prec, const void* src, const Geom& g,
                                       bool full, int parity, int nrhs, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
     const int np = full ? 2 : 1;
     dim3 grid((g.Vh + kBlock - 1) / kBlock, nrhs * np);
     const char* n = static_cast<const char*>(src);
     if (dst_prec == LQ_F64) {
-        LQ_DP_SWITCH(src_prec, (spinor_from_native_kernel<DP, LQ_F64><<<grid, kBlock, 0, st>>>(dst, n, g, full, parity, np)))
+        LQ_DP_SWITCH(src_prec, e = launch_conversion(spinor_from_native_kernel<DP, LQ_F64>, grid, st, dst, n, g, full, parity, np))
     } else {
-        LQ_DP_SWITCH(src_prec, (spinor_from_native_kernel<DP, LQ_F32><<<grid, kBlock, 0, st>>>(dst, n, g, full, parity, np)))
+        LQ_DP_SWITCH(src_prec, e = launch_conversion(spinor_from_native_kernel<DP, LQ_F32>, grid, st, dst, n, g, full, parity, np))
     }
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_native_convert(int dst_prec, void* dst, int src_prec, const void* src, int Vh, int nblocks,
