@@ -17,7 +17,7 @@
 // A thread owns one (site, 16-byte plane) and sweeps twice over the Ls slices:
 // once for z_end, once to write y.  Each slice is read before it is written, so
 // the call may run in place.  O(Ls) work per component, bandwidth-bound, or, on
-// lattices that fit L2, bound by the latency of one slice after the other: both
+// lattices that fit L2, bound by the latency of one slice after the other: the Moebius
 // kernels therefore load kBatch slices at a time (a load may not move above the
 // store of the slice before, as in and out may be one field).  12^3 x 24 x 11, FP32: the
 // combination 13.6 -> 7 us, the even-odd Moebius operator 77 -> 61 us (4, 6 or 8 alike).
@@ -74,16 +74,19 @@ __global__ void __launch_bounds__(256) m5inv_kernel(char* out, const char* in, i
     auto slice = [&](int j) { return fwd ? j : Ls - 1 - j; };
     V z = {};
     T w = g;
-    V x[kBatch];
+    // The Shamir inverse, between two hops, keeps to one slice at a time: with more registers its blocks leave
+    // the next hop's early blocks an uneven spread over the SMs (16 x 10 x 8 x 10, 16 slices: 33.3 -> 38.6 us).
+    constexpr int KB = WITH_B ? kBatch : 1;
+    V x[KB];
     auto load = [&](int j0) {
 #pragma unroll
-        for (int b = 0; b < kBatch; ++b)
+        for (int b = 0; b < KB; ++b)
             if (j0 + b < Ls) x[b] = *reinterpret_cast<const V*>(src + (size_t)slice(j0 + b) * in_stride);
     };
-    for (int j0 = 0; j0 < Ls; j0 += kBatch) {
+    for (int j0 = 0; j0 < Ls; j0 += KB) {
         load(j0);
 #pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
+        for (int b = 0; b < KB; ++b) {
             if (j0 + b >= Ls) break;
             z = axpby4<V, T>(pc, x[b], g, z);
             if (WITH_B && j0 + b + 1 < Ls) w *= g;
@@ -96,10 +99,10 @@ __global__ void __launch_bounds__(256) m5inv_kernel(char* out, const char* in, i
     T cw = -(T)mf_d * c5;  // S across the wall: -mf
     z = V{};
     w = g;
-    for (int j0 = 0; j0 < Ls; j0 += kBatch) {
-        if (j0 > 0 || Ls > kBatch) load(j0);  // (else the first sweep's loads are still here)
+    for (int j0 = 0; j0 < Ls; j0 += KB) {
+        if (j0 > 0 || Ls > KB) load(j0);  // (else the first sweep's loads are still here)
 #pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
+        for (int b = 0; b < KB; ++b) {
             if (j0 + b >= Ls) break;
             const int s = slice(j0 + b);
             z = axpby4<V, T>(pc, x[b], g, z);
