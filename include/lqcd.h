@@ -143,8 +143,9 @@ int lq_convert(lq_handle *h, void *dst, int dst_fmt, const void *src, int src_fm
  * (converted to native and back inside the call, using handle workspace), or
  * LQ_NATIVE | p (streamed directly).  FP32, FP16 and BF16 fields compute in FP32
  * with links stored in the same precision.  FP64 fields compute in FP64, or, with
- * links that are SU(3) (entries up to 1, rows and columns of 1-norm up to 2.75, which
- * lq_create checks), form the hopping sums in 64-bit fixed point: exact products and
+ * links of the scale of SU(3) (entries up to 1, rows and columns of 1-norm up to 2.75
+ * and with a real of at least 1/4, or links that are zero, which lq_create checks with
+ * one pass over the links), form the hopping sums in 64-bit fixed point: exact products and
  * sums to 2^-56 of the largest component of the site's 8 neighbours, rounded to FP64
  * once.
  */

@@ -223,24 +223,38 @@ __device__ __forceinline__ float abs_f32(double v) {
 }
 __device__ __forceinline__ float abs_f32(float v) { return fabsf(v) < 2.0f ? fabsf(v) : 4.0f; }
 
-// The links that the fixed-point FP64 hop cannot take: its sums are bounded for entries up to 1
-// and rows and columns of 1-norm up to 2.75 (SU(3): sqrt 6).
+__device__ __forceinline__ bool nonzero(double v) {
+    return (((unsigned)__double2hiint(v) << 1) | (unsigned)__double2loint(v)) != 0;
+}
+__device__ __forceinline__ bool nonzero(float v) { return v != 0.0f; }
+
+// The links that the fixed-point FP64 hop cannot take.  Its sums are bounded for entries up to 1 and
+// rows and columns of 1-norm up to 2.75 (SU(3): sqrt 6), and it keeps an entry to 2^-59, which is
+// enough where every row and column holds a real of at least 1/4 (SU(3): 1/sqrt 6) and loses
+// digits for links of a smaller scale.  A link that is exactly zero (an open boundary) is exact.
 template <typename T>
 __global__ void link_fixed_check_kernel(const T* src, long nlinks, unsigned* bad) {
     unsigned n = 0;
     for (long l = (long)blockIdx.x * blockDim.x + threadIdx.x; l < nlinks; l += (long)gridDim.x * blockDim.x) {
-        float row[3] = {}, col[3] = {};
-        bool ok = true;
+        float row[3] = {}, col[3] = {}, row_max[3] = {}, col_max[3] = {};
+        bool ok = true, zero = true;
 #pragma unroll
         for (int k = 0; k < 18; ++k) {
-            const float f = abs_f32(src[l * 18 + k]);
+            const T v = src[l * 18 + k];
+            const float f = abs_f32(v);
+            zero = zero && !nonzero(v);
             ok = ok && f <= 1.000001f;
             row[k / 6] += f;
             col[k / 2 % 3] += f;
+            row_max[k / 6] = fmaxf(row_max[k / 6], f);
+            col_max[k / 2 % 3] = fmaxf(col_max[k / 2 % 3], f);
         }
 #pragma unroll
-        for (int k = 0; k < 3; ++k) ok = ok && row[k] <= 2.75f && col[k] <= 2.75f;
-        n += ok ? 0 : 1;
+        for (int k = 0; k < 3; ++k) {
+            ok = ok && row[k] <= 2.75f && col[k] <= 2.75f;
+            ok = ok && row_max[k] >= 0.25f && col_max[k] >= 0.25f;
+        }
+        n += ok || zero ? 0 : 1;
     }
     if (n) atomicAdd(bad, n);
 }
