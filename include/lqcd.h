@@ -145,9 +145,11 @@ int lq_convert(lq_handle *h, void *dst, int dst_fmt, const void *src, int src_fm
  * with links stored in the same precision.  FP64 fields compute in FP64, or, with
  * links of the scale of SU(3) (entries up to 1, rows and columns of 1-norm up to 2.75
  * and with a real of at least 1/4, or links that are zero, which lq_create checks with
- * one pass over the links), form the hopping sums in 64-bit fixed point: exact products and
- * sums to 2^-56 of the largest component of the site's 8 neighbours, rounded to FP64
- * once.
+ * one pass over the links), form the hopping sums in 64-bit fixed point.  A fixed-point
+ * sum is used where, with S the sum of |U| |h| over directions and colours (h: the
+ * projected neighbour), its error is at most 1.8 2^-53 S as a standard deviation (95 2^-53 S
+ * in the worst case; FP64 sums: 15); a site with a component for which that does not hold
+ * takes FP64 sums.  Largest error measured: 3.2 2^-53 S, FP64 4.0.
  */
 int dslash_apply(lq_handle *h, void *out, const void *in, int fmt, int parity, int nrhs, void *stream);
 int dslash_dag_apply(lq_handle *h, void *out, const void *in, int fmt, int parity, int nrhs, void *stream);

@@ -113,6 +113,8 @@ static HopArgs base_args(lq_handle* h, const char* links, size_t lb) {
     a.skip = h->skip;
     a.skip_stride = h->skip_stride;
     a.fixed = h->fixed64;
+    a.u_sm = h->U_sm;
+    a.u_f32 = h->U_prec == LQ_F32;
     a.mma = h->hop_kernel == LQ_HOP_TENSOR_CORES ? 1 : 0;
     return a;
 }

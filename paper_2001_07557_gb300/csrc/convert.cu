@@ -34,12 +34,6 @@ __device__ __forceinline__ void load_sm(const void* base, size_t site, cplx<T> (
     }
 }
 
-__device__ __forceinline__ size_t lexi_of(const Geom& g, int cb, int p) {
-    int x[4];
-    cb_coords(g, cb, p, x);
-    return (size_t)x[0] + (size_t)g.L[0] * (x[1] + (size_t)g.L[1] * (x[2] + (size_t)g.L[2] * x[3]));
-}
-
 constexpr int kBlock = 128;
 
 // Arithmetic of a conversion: FP64 only where both sides are FP64 or one is and the other holds

@@ -14,19 +14,27 @@
 //   * links are packed once as u 2^58 = hi * 2^30 + lo (|lo| <= 2^29);
 //   * a real product is three multiply-adds: hi*hi, and hi*lo + lo*hi into a
 //     second 64-bit sum that is rounded in at the end of each dot product
-//     (lo*lo, below 2^-57 of the block, is dropped);
+//     (lo*lo, at most 2^-57 of the block, is dropped);
 //   * the 24 sums over 8 directions are 64-bit integers in units of 2^(B-57).
 //     A neighbour larger than 2^B moves the sums to its exponent.
 //
-// Precision: the sums carry 57 bits below the largest neighbour component (56 where the
-// headroom of the block exponent is used), against the 53 bits of each FP64 partial sum.
-// Against sums in quadruple precision the hop on 8^4 (random and smooth links) is 5.8e-17 off,
-// norm-wise, and 1.5e-16 with the FP64 kernel.  What is not finite, beyond 2^976 or below
-// 2^-894 takes the FP64 sums of slow_site.
+// Precision: a sum of 48 products is 2^-56.2 of the block off (standard deviation, exact-integer
+// restatement on Gaussian neighbours; worst case 190 2^-58: 96 from lo*lo, 48 from links kept to 2^-59,
+// 22 from spinors cut at 2^-59, 24 from rounding 8 products and moving the sums).  The block is 1 to
+// 4 times the largest neighbour component.  An FP64 sum is some u = 2^-53 times sum |U| |h| off (worst
+// case 15 u).  So that no component has less precision than in FP64, a sum is kept only if its terms
+// add up to 1/16 of the block (sizes are summed along with the terms), which is then 1.8 u of it (95 u in
+// the worst case); a site with any other goes to slow_site, which sums in FP64 from the links the
+// handle was given.  Largest error of a component over
+// sum |U| |h|, on dense fields, sources, fields whose spins, colours or sites differ by powers of ten, and
+// links near 1: 3.2 u here, 4.0 u in FP64; 7.4 u with a line at 1/32 and 3.2 u with one at 1/8.
+// Norm-wise the hop on 8^4 (random and smooth links) is 5.8e-17 off, and 1.5e-16 with the FP64 kernel.
+// What is not finite or beyond 2^976 takes slow_site too, and what is below 2^-894, as it is small
+// beside the least block.
 //
 // It needs links with |u| <= 1 and rows and columns of 1-norm <= 2.75 (SU(3): <= 2.45), which
-// bounds every sum below 2^63 (link_fixed_check_kernel, when a handle is made); other links
-// keep the FP64 kernel.
+// bounds every sum below 2^63, and with a real of at least 1/4 (link_fixed_check_kernel, when a handle is
+// made); other links keep the FP64 kernel.
 //
 // Layout: two threads a site, one for each spin of the half spinors; lanes 0-15 and 16-31 of a
 // warp share 16 sites.  A site's neighbour spinor (192 B) and link (144 B) come by cp.async into
@@ -36,10 +44,12 @@
 // code kept warps waiting for instructions (240 us); one looped body with run-time directions
 // executed 10,800 instructions a site where this takes 8,900 (236 against 215 us).
 //
-// Measured: D on 32^3 x 16 (as many sites as an even-odd hop of 32^4): 0.90 ms in FP64, 0.215 ms
+// Measured: D on 32^3 x 16 (as many sites as an even-odd hop of 32^4): 0.92 ms in FP64, 0.214 ms
 // here; its bytes take 0.12 ms.  What bounds it is the integer pipes: without its products,
 // conversions and sums the kernel takes 0.123 ms; the multiplier is busy 64 % of the time, the
-// ALU 44 %, with warps waiting on fixed latencies (ncu).
+// ALU 44 %, with warps waiting on fixed latencies (ncu).  The sizes cost 1.3 % of a dense field's
+// time.  Where every site takes slow_site (one spin and colour alone on every site): 0.97 ms; the
+// zero field 0.234, a point source 0.267.
 #pragma once
 
 #include <cuda_pipeline.h>
@@ -51,44 +61,75 @@ namespace lq {
 
 constexpr int kFixEmin = 128;    // biased exponents the block may have
 constexpr int kFixEmax = 2000;
+// A sum is kept where its terms, one for each direction, add up to this many 2^-10 of the block
+// (larger of the real and the imaginary part of each); others are formed in FP64.  1/16: see above; plain
+// FP64 CG from a point source on 16^3 x 32 takes 23.2 ms, 20.4 with a line at 1/32, 30.8 at 1/8 and
+// 60.9 with the FP64 kernel.
+constexpr int kFixWeak = 64;
 
-// ------------------------------------------------------------------- links
+// ------------------------------------------------- sites summed in FP64
 
-// entry of a fixed-point link (fix_link_entry)
-__device__ __forceinline__ double fix_link_value(int hi, int lo) {
-    return (double)(((long long)hi << 30) + lo) * 3.469446951953614189e-18;  // 2^-58
+// z, negated for a set flag
+__device__ __forceinline__ cplx<double> flip_sign(cplx<double> z, bool f) {
+    const int m = f ? (int)0x80000000 : 0;
+    return {__hiloint2double(__double2hiint(z.re) ^ m, __double2loint(z.re)),
+            __hiloint2double(__double2hiint(z.im) ^ m, __double2loint(z.im))};
 }
 
-// The hop sums of one site in FP64, from the fixed-point links: for neighbours that are not
-// finite or out of the fixed-point range.  out: 24 doubles, NT * 2 apart by pairs.
+// The hop sums of one site with the FP64 unit, from the links as the handle was given them: for
+// sums that the fixed-point ones do not hold well enough, and neighbours that are not finite or out
+// of their range.  Each of the site's two threads does the half of its spin, so that a warp's
+// instructions do as much as those of the FP64 kernel.  To shared memory, NT apart: in s the
+// sums of spin s and then those of spin 2 + s without the other thread's part, in l that part.
 template <bool DAG, int NT>
-__device__ __noinline__ void slow_site(const HopArgs& a, int p, const char* in, int i, const int* nbr, int flips,
-                                       double2* out) {
-    cplx<double> acc[12];
+__device__ __noinline__ void slow_site(const HopArgs& a, int p, int spin, const char* in, int i, const int* nbr,
+                                       int flips, double2* s, double2* l) {
+    cplx<double> up[3], lx[3], ly[3];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = {0.0, 0.0};
-    const char* Lp = a.links + (size_t)(p * 4) * a.link_block;
-    const char* Lq = a.links + (size_t)((1 - p) * 4) * a.link_block;
+    for (int c = 0; c < 3; ++c) up[c] = lx[c] = ly[c] = {0.0, 0.0};
+    const size_t own = lexi_of(a.g, i, p);
     auto dir = [&](auto dtag) {
         constexpr int D = decltype(dtag)::value, MU = D >> 1;
         constexpr bool FWD = (D & 1) == 0;
         constexpr int S = (FWD == DAG) ? 1 : -1;
         const int n = nbr[D * NT];
-        cplx<double> s[12], h[6], u[9], uh[6];
-        load_spinor<LQ_F64, double>(in, a.g.Vh, n, s);
-        project<MU, S>(s, h);
-        const int4* lk = reinterpret_cast<const int4*>((FWD ? Lp : Lq) + (size_t)MU * a.link_block);
+        const double2* q = reinterpret_cast<const double2*>(in) + n;
+        const size_t link = ((FWD ? own : lexi_of(a.g, n, 1 - p)) * 4 + MU) * 9;
+        cplx<double> h[3], u[9];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {  // the projector, as in project()
+            const double2 x = __ldg(q + (size_t)(3 * spin + c) * a.g.Vh);
+            const double2 y = __ldg(q + (size_t)((MU < 2 ? 9 - 3 * spin : 6 + 3 * spin) + c) * a.g.Vh);
+            cplx<double> z = {y.x, y.y};
+            if constexpr (MU == 0) z = cneg(cmul_i(z));
+            else if constexpr (MU == 1) z = flip_sign(z, spin == 0);
+            else if constexpr (MU == 2) z = flip_sign(cmul_i(z), spin == 0);
+            h[c] = flip_sign(cadds<S>(cplx<double>{x.x, x.y}, z), (flips >> D) & 1);
+        }
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            const int4 v = __ldg(lk + (size_t)k * a.g.Vh + (FWD ? i : n));
-            u[k] = {fix_link_value(v.y, v.x), fix_link_value(v.w, v.z)};
+            if (a.u_f32) {
+                const float2 v = __ldg(reinterpret_cast<const float2*>(a.u_sm) + link + k);
+                u[k] = {widen(v.x), widen(v.y)};
+            } else {
+                const double2 v = __ldg(reinterpret_cast<const double2*>(a.u_sm) + link + k);
+                u[k] = {v.x, v.y};
+            }
         }
-        if ((flips >> D) & 1) {
 #pragma unroll
-            for (int k = 0; k < 6; ++k) h[k] = cneg(h[k]);
+        for (int c = 0; c < 3; ++c) {  // reconstruct_add()
+            cplx<double> w = {0.0, 0.0};
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                if constexpr (FWD) cmac(w, u[3 * c + j], h[j]);
+                else cmac_conj(w, u[3 * j + c], h[j]);
+            }
+            up[c] = cadd(up[c], w);
+            if constexpr (MU == 0) lx[c] = cadds<S>(lx[c], cmul_i(w));
+            else if constexpr (MU == 1) lx[c] = cadds<S>(lx[c], flip_sign(w, spin == 0));
+            else if constexpr (MU == 2) ly[c] = cadds<S>(ly[c], flip_sign(cmul_i(w), spin == 1));
+            else ly[c] = cadds<S>(ly[c], w);
         }
-        su3_mul<!FWD>(u, h, uh);
-        reconstruct_add<MU, S>(acc, uh);
     };
     dir(std::integral_constant<int, 0>());
     dir(std::integral_constant<int, 1>());
@@ -99,7 +140,40 @@ __device__ __noinline__ void slow_site(const HopArgs& a, int p, const char* in, 
     dir(std::integral_constant<int, 6>());
     dir(std::integral_constant<int, 7>());
 #pragma unroll
-    for (int k = 0; k < 12; ++k) out[k * NT] = make_double2(acc[k].re, acc[k].im);
+    for (int c = 0; c < 3; ++c) {
+        s[(6 * spin + c) * NT] = make_double2(up[c].re, up[c].im);
+        s[(6 * spin + 3 + c) * NT] = make_double2(ly[c].re, ly[c].im);
+        l[(3 * spin + c) * NT] = make_double2(lx[c].re, lx[c].im);
+    }
+}
+
+// Do the half spinors of spin `spin` hold anything but zeros?  Nonzero x for the x and y
+// directions, y for z and t (there after the projection in FP64, as in the kernel).
+template <bool DAG, int NT>
+__device__ __noinline__ uint2 nonzero_halves(const HopArgs& a, int spin, const char* in, const int* nbr) {
+    uint2 seen = {0, 0};
+    auto bits = [](uint4 v) { return v.x | v.z | (v.y | v.w) << 1; };
+    for (int d = 0; d < 8; ++d) {
+        const uint4* q = reinterpret_cast<const uint4*>(in) + nbr[d * NT];
+        const int o = d < 4 ? 9 - 3 * spin : 6 + 3 * spin;
+        const bool minus = ((d & 1) == 0) != DAG;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            uint4 x = __ldg(q + (size_t)(3 * spin + c) * a.g.Vh);
+            const uint4 y = __ldg(q + (size_t)(o + c) * a.g.Vh);
+            if (d < 4) {
+                seen.x |= bits(x) | bits(y);
+            } else if (d < 6) {
+                seen.y |= bits(x) | bits(y);
+            } else {
+                const uint32_t f = minus ? 0x80000000u : 0;
+                const uint2 re = words(value(make_uint2(x.x, x.y)) + value(make_uint2(y.x, y.y ^ f)));
+                const uint2 im = words(value(make_uint2(x.z, x.w)) + value(make_uint2(y.z, y.w ^ f)));
+                seen.y |= bits(make_uint4(re.x, re.y, im.x, im.y));
+            }
+        }
+    }
+    return seen;
 }
 
 // ------------------------------------------------------------------ kernel
@@ -115,7 +189,7 @@ struct FixSmem {
 };
 
 template <bool DAG, int EPI, bool RED>
-__global__ void __launch_bounds__(kFixThreads, 3) wilson_hop_fixed_kernel(const HopArgs a) {
+__global__ void __launch_bounds__(kFixThreads, 3) wilson_hop_fixed_kernel(const __grid_constant__ HopArgs a) {
     constexpr int NT = kHopThreads, PL = FixSmem::PL;
     extern __shared__ __align__(16) unsigned char smem[];
     // lane 16 s + j: spin s of the half spinors of the warp's site j
@@ -187,13 +261,16 @@ __global__ void __launch_bounds__(kFixThreads, 3) wilson_hop_fixed_kernel(const 
         __syncwarp();
     };
 
-    // sums over directions, [2 c + {re, im}]: up of spin s; lx and ly of the lower spins, lx (from
-    // x and y hops) of spin 2 + (1 - s), ly (z and t) of spin 2 + s
-    long long up[6], lx[6], ly[6];
+    // sums over directions, [2 c + {re, im}]: up of spin s, low of a lower spin: 2 + (1 - s) for the x
+    // and y hops, after which the site's threads exchange theirs, and 2 + s from then on
+    long long up[6], low[6];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) up[k] = lx[k] = ly[k] = 0;
+    for (int k = 0; k < 6; ++k) up[k] = low[k] = 0;
     int eb = 0;  // the block's biased exponent: |neighbour components| < 2^(eb - 1022)
     bool slow = false;
+    // sums over directions of the larger part of each term of colour c in units of 2^-10 of the block (at
+    // most 8 * 5.5 * 2^10): for up in the upper, for low in the lower 16 bits (x and y: both the lower)
+    uint32_t size[3] = {0, 0, 0};
 
     issue_spinor(in, nbr[NT]);
     __pipeline_commit();
@@ -253,9 +330,10 @@ __global__ void __launch_bounds__(kFixThreads, 3) wilson_hop_fixed_kernel(const 
 #pragma unroll
                     for (int k = 0; k < 6; ++k) {
                         up[k] = sar64(up[k], n);
-                        lx[k] = sar64(lx[k], n);
-                        ly[k] = sar64(ly[k], n);
+                        low[k] = sar64(low[k], n);
                     }
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) size[c] = shr32(size[c], 16 + n) << 16 | shr32(size[c] & 0xffffu, n);
                     eb = to;
                     slow = slow || to > kFixEmax;
                 }
@@ -304,30 +382,34 @@ __global__ void __launch_bounds__(kFixThreads, 3) wilson_hop_fixed_kernel(const 
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const long long re = w[2 * c], im = w[2 * c + 1];
+                const uint32_t part = (uint32_t)max(abs((int)(re >> 32)), abs((int)(im >> 32)));
+                size[c] += (part >> 15) * (MU < 2 ? 1 : 0x10001);
                 up[2 * c] += re;
                 up[2 * c + 1] = im - up[2 * c + 1];
                 if constexpr (MU == 0) {
-                    lx[2 * c] -= im;
-                    lx[2 * c + 1] = re - lx[2 * c + 1];
+                    low[2 * c] -= im;
+                    low[2 * c + 1] = re - low[2 * c + 1];
                 } else if constexpr (MU == 1) {
-                    lx[2 * c] = ((re ^ n) - n) - lx[2 * c];
-                    lx[2 * c + 1] += (im ^ n) - n;
+                    low[2 * c] = ((re ^ n) - n) - low[2 * c];
+                    low[2 * c + 1] += (im ^ n) - n;
                 } else if constexpr (MU == 2) {
-                    ly[2 * c] -= (im ^ n) - n;
-                    ly[2 * c + 1] = ((re ^ n) - n) - ly[2 * c + 1];
+                    low[2 * c] -= (im ^ n) - n;
+                    low[2 * c + 1] = ((re ^ n) - n) - low[2 * c + 1];
                 } else {
-                    ly[2 * c] = re - ly[2 * c];
-                    ly[2 * c + 1] += im;
+                    low[2 * c] = re - low[2 * c];
+                    low[2 * c + 1] += im;
                 }
             }
         }
     };
     dimension(std::integral_constant<int, 0>());
     dimension(std::integral_constant<int, 1>());
+#pragma unroll
+    for (int k = 0; k < 6; ++k) low[k] = __shfl_xor_sync(0xffffffffu, low[k], 16);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) size[c] = size[c] << 16 | __shfl_xor_sync(0xffffffffu, size[c], 16);
     dimension(std::integral_constant<int, 2>());
     dimension(std::integral_constant<int, 3>());
-#pragma unroll
-    for (int k = 0; k < 6; ++k) ly[k] += __shfl_xor_sync(0xffffffffu, lx[k], 16);
 
     // c_hop, and S of the forward projectors for the lower spins; a power of two (all but the second
     // hop of the Schur complement) goes into the exponent
@@ -341,44 +423,45 @@ __global__ void __launch_bounds__(kFixThreads, 3) wilson_hop_fixed_kernel(const 
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
         o[k] = fix_to_double(up[k], ef, fu);
-        o[6 + k] = fix_to_double(ly[k], ef, fl);
+        o[6 + k] = fix_to_double(low[k], ef, fl);
     }
     if (!pow2) {
 #pragma unroll
         for (int k = 0; k < 12; ++k) o[k] *= ch;
     }
-    // neighbours that are all subnormal or tiny (the block exponent 0 or held at kFixEmin), and those
-    // out of range above, take the FP64 sums, by way of the site's spinor slot.  Neighbours that are
-    // all exactly zero do not, as their sums are zero already: they are told apart by reading them once
-    // more (32^3 x 16, a point source: 2488 us with FP64 sums everywhere but near the source,
-    // 233 us here; a dense field takes 221 us, and 227 us with a flag kept in the loop).
-    if (__any_sync(0xffffffffu, slow || eb <= kFixEmin)) {
-        uint32_t seen = 0;
-        if (slow || eb <= kFixEmin) {
-            for (int d = 0; d < 8; ++d) {
-                const char* q = in + (size_t)(6 * spin) * plane + (size_t)nbr[d * NT] * 16;
+    // Where the terms of a sum are small beside the block (a neighbour of much larger other spins,
+    // colours or sites, links with small entries, neighbours that are subnormal or out of the fixed-point
+    // range), the block's bits are too few for it: the site takes the FP64 sums.  Sums of exact zeros
+    // (around sources) are zero already; they are told apart by reading the neighbours once more.
+    bool weak_up = false, weak_low = false;
 #pragma unroll
-                for (int k = 0; k < 6; ++k) {
-                    const uint4 v = __ldg(reinterpret_cast<const uint4*>(q + k * plane));
-                    seen |= v.x | v.z | (v.y | v.w) << 1;
-                }
-            }
-        }
-        seen |= __shfl_xor_sync(0xffffffffu, seen, 16);
-        const bool mine = seen != 0;  // the same for a site's two threads
+    for (int c = 0; c < 3; ++c) {
+        weak_up |= size[c] >> 16 < kFixWeak;
+        weak_low |= (size[c] & 0xffffu) < kFixWeak;
+    }
+    bool mine = slow || weak_up || weak_low;
+    if (__any_sync(0xffffffffu, mine)) {
+        mine = __shfl_xor_sync(0xffffffffu, mine, 16) || mine;  // the same for a site's two threads
+        uint2 seen = {0, 0};
+        if (mine) seen = nonzero_halves<DAG, NT>(a, spin, in, nbr);
+        const uint32_t seen_xy = __shfl_xor_sync(0xffffffffu, seen.x, 16);
+        mine = slow || (weak_up && (seen.x | seen.y)) || (weak_low && (seen_xy | seen.y));
+        mine = __shfl_xor_sync(0xffffffffu, mine, 16) || mine;
         __pipeline_wait_prior(0);
         __syncwarp();
         double2* v = reinterpret_cast<double2*>(sp);
-        if (mine && spin == 0) slow_site<DAG, NT>(a, p, in, i, nbr, flips, v);
+        double2* x = reinterpret_cast<double2*>(lk);
+        if (mine) slow_site<DAG, NT>(a, p, spin, in, i, nbr, flips, v, x);
         __syncwarp();
         if (mine) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const double2 b = v[(3 * spin + c) * NT], l = v[(6 + 3 * spin + c) * NT];
+                const double2 b = v[(6 * spin + c) * NT], l = v[(6 * spin + 3 + c) * NT];
+                const double2 m = x[(3 - 3 * spin + c) * NT];
                 o[2 * c] = ch * b.x;
                 o[2 * c + 1] = ch * b.y;
-                o[6 + 2 * c] = ch * l.x;
-                o[6 + 2 * c + 1] = ch * l.y;
+                o[6 + 2 * c] = ch * (l.x + m.x);
+                o[6 + 2 * c + 1] = ch * (l.y + m.y);
             }
         }
         __syncwarp();

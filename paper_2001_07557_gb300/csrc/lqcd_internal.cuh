@@ -53,6 +53,13 @@ __device__ __forceinline__ void cb_coords(const Geom& g, int cb, int p, int x[4]
     x[0] = 2 * xh + ((p + x[1] + x[2] + x[3]) & 1);
 }
 
+// Its lexicographic index, x0 fastest.
+__device__ __forceinline__ size_t lexi_of(const Geom& g, int cb, int p) {
+    int x[4];
+    cb_coords(g, cb, p, x);
+    return (size_t)x[0] + (size_t)g.L[0] * (x[1] + (size_t)g.L[1] * (x[2] + (size_t)g.L[2] * x[3]));
+}
+
 // Device-resident CG scalars of one right-hand side.
 struct CgScalars {
     double rr;     // |r|^2

@@ -37,6 +37,8 @@ struct HopArgs {
     // its SU(3) products on the tensor cores (hop_mma.cuh); 0: CUDA cores only
     int mma;
     int fixed;  // FP64: the links are the fixed-point ones of hop_fixed.cuh
+    const void* u_sm;  // and these the site-major ones that the handle was given, FP64 or (u_f32) FP32
+    int u_f32;
     const int* skip;  // optional per-rhs flags (skip[rhs * skip_stride]): a set flag ends the block at once
     int skip_stride;
     // optional fused |out|^2 per right-hand side (one group for the domain wall):
