@@ -407,10 +407,12 @@ int lq_face_unpack(lq_handle *h, void *dst, int t_dst, const void *wire, int fmt
  *     (LQ_ERR_LAYOUT otherwise).  The caller owns all three.
  *   - C may be the same pointer as A or as B (the product is formed in place
  *     tile by tile); any other overlap is LQ_ERR_ARG.
- *   - FP64 matrices of the scale of SU(3) (every real at most 1, every row of A
- *     and column of B with a real of at least 1/4) are multiplied in 64-bit fixed
- *     point: an entry is a sum good to 2^-57, rounded to FP64 once.  Others are
- *     multiplied in FP64, FP32 ones in FP32.
+ *   - FP64 matrices whose reals are at most 1 are multiplied in 64-bit fixed point where
+ *     that is as accurate as FP64: a real of C comes from it where S, the sum of the
+ *     absolute values of its six products, is at least 1/32, which makes its rounding
+ *     error before the last rounding at most 0.87 2^-53 S as a standard deviation
+ *     (12.5 2^-53 S in the worst case; FP64 sums: 6).  Other reals are formed in FP64,
+ *     FP32 matrices are multiplied in FP32.
  *   - n = 0 is a no-op; n < 0 or a null pointer with n > 0 is LQ_ERR_ARG.
  *   - Asynchronous on `stream`.  No handle is needed and nothing is allocated.
  * Tiles of A and B move to shared memory by bulk asynchronous copies that

@@ -10,12 +10,13 @@
 //     the copies of the next tile are in flight while this one is multiplied;
 //   * thread t multiplies matrix t of the tile.  Its shared-memory reads have
 //     a stride of 72 or 144 bytes, which touches every bank once per phase;
-//   * the products go to one of two output buffers, which one thread writes
-//     back with a bulk store.
+//   * the products go to one of two output buffers (FP64: over the tile of A),
+//     which one thread writes back with a bulk store.
 // FP32 is bound by HBM bandwidth (216 bytes and 198 flop per matrix).  FP64
 // would be bound by the FP64 units: 198 flop take longer at GB300's FP64 rate
 // than its 432 bytes take to move.  Matrices of SU(3) scale are therefore
-// multiplied in fixed point on the integer units.  Every barrier wait is bounded; a wait that runs
+// multiplied in fixed point on the integer units, but for the few reals that
+// these would give less precisely.  Every barrier wait is bounded; a wait that runs
 // out is counted in g_wait_timeouts and its block stops.  Before it returns,
 // the block waits (bounded again) for the copies it issued into its other
 // stage, and for its bulk stores, so that no copy into its shared memory is
@@ -29,6 +30,7 @@
 
 #include "fixed.cuh"
 #include "lqcd.h"
+#include "lqcd_internal.cuh"
 #include "trace.h"
 
 namespace lq {
@@ -116,48 +118,136 @@ __device__ __forceinline__ void su3_product(const T2 (&a)[9], const T2 (&b)[9], 
     }
 }
 
-// The FP64 product in fixed point (fixed.cuh), for two matrices whose scale is that of SU(3):
-// every real at most 1 (and 2^-20), every row of A and column of B with a real of at least 1/4,
-// as unitary ones have (1/sqrt 6).  The block exponent is then the same for all, 2^0, and an
-// entry of C is rounded once from a sum exact to 2^-57.  False for any other pair, which the
-// FP64 unit multiplies.  Against sums in quadruple precision the products of smooth links
-// (exp(0.3 i H)) are 3.9e-17 off, norm-wise, and 7.4e-17 with the FP64 unit.  108 FP64 instructions
-// at 77 clocks a warp and SM sub-partition compare with about 1,400 integer ones here.  48^4: 991 us in FP64, 511 us with two blocks an SM and
-// output buffers, 418 us with three blocks and in place (0.81 of the HBM time of its bytes;
-// four blocks of one stage 434 us).
+// The FP64 product in fixed point (fixed.cuh): every real of A and B (at most 1) is cut to a
+// multiple of 2^-59, and a real of C is a sum of six products, lo lo parts left out, rounded once.
+// Before that rounding it is 2^-58.2 off as a standard deviation (exact-integer restatement on random and
+// smooth links; worst case 12.5 2^-58, for SU(3) 9 2^-58).  An FP64 sum is some u = 2^-53 times S off,
+// the sum of the six products' absolute values (worst case 6 u S).  So that no real has less precision
+// than in FP64, those with S < 1/32 (there 0.87 u S, worst case 12.5) are formed with the FP64 unit, and so
+// are all of a pair that holds a real above 1 or more than kSu3Few such.  Largest error over S measured,
+// on random and smooth links exp(i eps H), eps 0.3 to 1e-6: 4.3 u, as with the FP64 unit alone
+// (a line at 1/64: 6.5 u, at 1/16 4.3 u).
+//
+// 108 FP64 instructions at 77 clocks a warp and SM sub-partition compare with about 1,600 integer and FP32
+// ones here.  48^4, smooth links: 991 us in FP64, 501 us here (467 where no sum is small, 421 without
+// the sums S; 0.68 of the HBM time of its bytes), with three blocks an SM and in place.  Where all of every pair
+// goes to the FP64 unit: 1027-1045 us; A = 1 and a smooth B 1049.  S after the fixed-point product: 483 and
+// 1190-1207 us.  lo lo included, which would allow a line at 1/64: 534 us.
+constexpr float kSu3Weak = 1.0f / 32;
+constexpr int kSu3Few = 8;  // weak reals of a pair that are formed one at a time, not with all of it
+
+__device__ __forceinline__ uint4 load16(const double2* p) { return *reinterpret_cast<const uint4*>(p); }
+
+// |x| of a double below 2 in FP32, from its high word; 2^-60 for anything smaller
+__device__ __forceinline__ float abs_cut(uint32_t hi) {
+    return __int_as_float(max((int)(hi & 0x7fffffffu) - 0x38000000, 0x04300000) << 3);
+}
+
+// One bit for each real of A B (2 (3 i + j) + {re, im}) with S < kSu3Weak; top: the largest
+// high word of the two matrices (max_hi).
+__device__ __forceinline__ uint32_t su3_weak(const double2* a, const double2* b, float& top) {
+    cplx<float> x[9];
+    top = 0.f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const uint4 v = load16(a + k);
+        top = max_hi(top, v.y, v.w);
+        x[k] = {abs_cut(v.y), abs_cut(v.w)};
+    }
+    uint32_t weak = 0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        cplx<float> y[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint4 v = load16(b + 3 * k + j);
+            top = max_hi(top, v.y, v.w);
+            y[k] = {abs_cut(v.y), abs_cut(v.w)};
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            cplx<float> s = {0.f, 0.f};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                fma2(s, x[3 * i + k].re, y[k]);
+                fma2(s, x[3 * i + k].im, cplx<float>{y[k].im, y[k].re});
+            }
+            if (s.re < kSu3Weak) weak |= 1u << 2 * (3 * i + j);
+            if (s.im < kSu3Weak) weak |= 2u << 2 * (3 * i + j);
+        }
+    }
+    return weak;
+}
+
+// Those of the reals in `weak` that have a product of two nonzero factors (the others are zero).
+__device__ __noinline__ uint32_t su3_nonzero(const double2* a, const double2* b, uint32_t weak) {
+    uint32_t ar = 0, ai = 0, br = 0, bi = 0;  // bit 3 i + k of A, 3 j + k of B
+    auto bit = [](uint32_t lo, uint32_t hi, int k) { return ((lo | hi << 1) != 0 ? 1u : 0u) << k; };
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const uint4 x = load16(a + k), y = load16(b + k);
+        const int t = 3 * (k % 3) + k / 3;
+        ar |= bit(x.x, x.y, k);
+        ai |= bit(x.z, x.w, k);
+        br |= bit(y.x, y.y, t);
+        bi |= bit(y.z, y.w, t);
+    }
+    uint32_t some = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const uint32_t xr = ar >> 3 * i, xi = ai >> 3 * i, yr = br >> 3 * j, yi = bi >> 3 * j;
+            if (((xr & yr) | (xi & yi)) & 7u) some |= 1u << 2 * (3 * i + j);
+            if (((xr & yi) | (xi & yr)) & 7u) some |= 2u << 2 * (3 * i + j);
+        }
+    }
+    return weak & some;
+}
+
+// Real e of A B with the FP64 unit.
+__device__ __noinline__ double su3_real(const double2* a, const double2* b, int e) {
+    const int i = e / 6, j = (e >> 1) % 3;
+    const bool im = e & 1;
+    double s = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const double2 x = a[3 * i + k], y = b[3 * k + j];
+        s = fma(x.x, im ? y.y : y.x, s);
+        s = fma(im ? x.y : -x.y, im ? y.x : y.y, s);
+    }
+    return s;
+}
+
 __device__ __forceinline__ bool su3_product_fixed(const double2* a, const double2* b, double2 (&c)[9]) {
     constexpr int EB = 1022;
     constexpr uint32_t E2 = ((uint32_t)EB << 21) + 0x1fffffu + (5u << 21);
-    constexpr int kOne = 0x3ff00001, kQuarter = 0x3fd00000;
+    constexpr int kOne = 0x3ff00001;
+    float top;
+    uint32_t weak = su3_weak(a, b, top);
+    if (!(__float_as_int(top) <= kOne)) return false;
+    if (__popc(weak) > kSu3Few) {
+        weak = su3_nonzero(a, b, weak);
+        if (__popc(weak) > kSu3Few) return false;
+    }
     Fix2 fa[18];
-    int top = 0, low = 0x7fffffff;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        float m = 0.f;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const uint2 re = words(a[3 * i + k].x), im = words(a[3 * i + k].y);
-            m = max_hi(m, re.y, im.y);
-            fa[6 * i + k] = fix_one(re, E2, 0);
-            fa[6 * i + 3 + k] = fix_one(im, E2, 0);
+            fa[6 * i + k] = fix_one(words(a[3 * i + k].x), E2, 0);
+            fa[6 * i + 3 + k] = fix_one(words(a[3 * i + k].y), E2, 0);
         }
-        top = max(top, __float_as_int(m));
-        low = min(low, __float_as_int(m));
     }
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        float m = 0.f;
         Fix2 x[6], y[6];  // column j as the factors of the real and of the imaginary part
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const uint2 re = words(b[3 * k + j].x), im = words(b[3 * k + j].y);
-            m = max_hi(m, re.y, im.y);
-            x[k] = y[3 + k] = fix_one(re, E2, 0);
-            y[k] = fix_one(im, E2, 0);
+            x[k] = y[3 + k] = fix_one(words(b[3 * k + j].x), E2, 0);
+            y[k] = fix_one(words(b[3 * k + j].y), E2, 0);
             x[3 + k] = {-y[k].hi, -y[k].lo};
         }
-        top = max(top, __float_as_int(m));
-        low = min(low, __float_as_int(m));
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const Fix2 u[6] = {fa[6 * i], fa[6 * i + 1], fa[6 * i + 2], fa[6 * i + 3], fa[6 * i + 4], fa[6 * i + 5]};
@@ -165,7 +255,17 @@ __device__ __forceinline__ bool su3_product_fixed(const double2* a, const double
             c[3 * i + j] = make_double2(fix_to_double(fix_dot(u, x), 1021, 0u), fix_to_double(fix_dot(u, y), 1021, 0u));
         }
     }
-    return top <= kOne && low >= kQuarter;
+    while (weak) {
+        const int e = __ffs((int)weak) - 1;
+        weak &= weak - 1;
+        const double v = su3_real(a, b, e);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            if (e == 2 * k) c[k].x = v;
+            if (e == 2 * k + 1) c[k].y = v;
+        }
+    }
+    return true;
 }
 
 // Shared memory: stage s holds the tile of A at 2*s*TB and of B at (2*s+1)*TB,
