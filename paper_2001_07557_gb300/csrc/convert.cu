@@ -263,14 +263,29 @@ __global__ void link_fixed_check_kernel(const T* src, long nlinks, unsigned* bad
     default: { constexpr int DP = LQ_BF16; BODY; } break;    \
     }
 
+// SMs of the current device, found once (0 where that fails)
+static int sm_count() {
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        return n;
+    }();
+    return sms;
+}
+
 // A conversion to or from site-major of up to four blocks per SM is launched as a programmatic
-// dependent: what it takes there is the launch (D on FP64 site-major fields, 4^4: 20.6 -> 16.0 us,
-// 8^3 x 16: 20.9 -> 17.8, 16^4: 51.6 -> 50.1).  A larger one is not: started beside the end of a hop,
+// dependent: what it takes there is the launch (D on FP64 site-major fields, 4^4: 20.5 -> 16.8 us,
+// 8^3 x 16: 20.9 -> 18.0, 16^4: 51.6 -> 50.1).  A larger one is not: started beside the end of a hop,
 // which holds most of L1 as shared memory, spinor_to_native_kernel lacks the L1 that gathers its 16-byte
 // reads into lines (32^4 FP64 after an FP32 hop: 163 -> 227 us for the two).
 template <typename... KArgs, typename... Args>
 static cudaError_t launch_conversion(void (*kern)(KArgs...), dim3 grid, cudaStream_t st, Args... args) {
-    if (grid.x * (size_t)grid.y <= 4 * 152) return launch_pdl(kern, grid, dim3(kBlock), 0, st, args...);
+    if (grid.x * (size_t)grid.y <= 4 * (size_t)sm_count())
+        return launch_pdl(kern, grid, dim3(kBlock), 0, st, args...);
     kern<<<grid, kBlock, 0, st>>>(args...);
     return cudaGetLastError();
 }
