@@ -309,6 +309,9 @@ typedef struct {
  * cg_solve: solve A x = b (A from cp->op) for cp->nrhs right-hand sides.
  * stats must point to cp->nrhs entries.  Returns LQ_OK when every right-hand
  * side reached tol, LQ_ERR_NOT_CONVERGED (x = best iterate) or another error.
+ * Its vectors stay with the handle.  Except in block CG, one of them (a second search
+ * direction per right-hand side, in the precision of the CG) is used where memory allows and
+ * given up where it does not; the iterates are the same.
  */
 int cg_solve(lq_handle *h, void *x, const void *b, const lq_cg_params *cp, lq_cg_stats *stats, void *stream);
 

@@ -30,13 +30,28 @@ cudaError_t launch_hop(int prec, const HopArgs& a, bool r12, bool dag, int epi, 
     }
 }
 
+// cudaMalloc; where there is no room, again without the one buffer that solves can do without
+// (cudaFree waits for the work that uses it, and a solve asks for it last)
+static cudaError_t handle_malloc(lq_handle* h, void** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    lq_handle::Buf& spare = h->ws[WS_CGP];
+    if (e != cudaSuccess && spare.ptr) {
+        cudaGetLastError();
+        cudaFree(spare.ptr);
+        spare.ptr = nullptr;
+        spare.bytes = 0;
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
 int ensure_ws(lq_handle* h, int k, size_t bytes, void** out) {
     lq_handle::Buf& b = h->ws[k];
     if (b.bytes < bytes) {
         if (b.ptr) cudaFree(b.ptr);
         b.ptr = nullptr;
         b.bytes = 0;
-        if (cudaMalloc(&b.ptr, bytes) != cudaSuccess) {
+        if (handle_malloc(h, &b.ptr, bytes) != cudaSuccess) {
             cudaGetLastError();
             b.ptr = nullptr;
             return LQ_ERR_NOMEM;
@@ -82,7 +97,7 @@ int get_links(lq_handle* h, int prec, const char** links, size_t* link_block, cu
     void*& L = h->links[prec][r12];
     const size_t lb = (size_t)link_site_bytes(prec, r12) * h->g.Vh;
     if (!L) {
-        if (cudaMalloc(&L, lb * 8) != cudaSuccess) {
+        if (handle_malloc(h, &L, lb * 8) != cudaSuccess) {
             cudaGetLastError();
             L = nullptr;
             return LQ_ERR_NOMEM;

@@ -127,6 +127,8 @@ __global__ void __launch_bounds__(kThreads) dot_kernel(VecRef a, VecRef b, int V
 // 195.5 -> 190.0 ms, mixed CG on 32^4 33.6 -> 33.0 ms).  The additions to x are those of a step at a time, in the same order.
 // pend holds the alphas whose alpha p is not in x yet; a right-hand side that finishes in the even
 // step leaves pend = {alpha, 0} to the odd one, and the next pair's even step clears it.
+// With one search direction (no memory for two) every step is an even one whose x is updated at
+// once, by cg_x_xpay_kernel with p0 = p1.
 
 // r -= alpha q ; rr_new = |r|^2 ; beta, convergence (per rhs)
 template <int PR, int PQ>

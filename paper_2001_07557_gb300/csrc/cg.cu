@@ -198,9 +198,6 @@ int run_cg(lq_handle* h, const OpGeom& og, const Ctl& c, int pp, const VecRef& e
     CgVecs v;
     int rc = cg_vectors(h, og, pr, pp, slot0, &v);
     if (rc) return rc;
-    void* pbuf;  // the second search direction
-    if ((rc = ensure_ws(h, WS_CGP, og.bytes(h, pp), &pbuf))) return rc;
-    const VecRef p2[2] = {v.p, og.ref(h, pbuf, pp)};
     const char* L;
     size_t lb;
     if ((rc = get_links(h, pp, &L, &lb, s))) return rc;  // pack before any capture
@@ -213,6 +210,13 @@ int run_cg(lq_handle* h, const OpGeom& og, const Ctl& c, int pp, const VecRef& e
         void* w;
         if ((rc = ensure_ws(h, WS_MOB, og.bytes(h, pp), &w))) return rc;
     }
+    // the second search direction, last, as any other buffer takes its place where memory is short
+    // (ensure_ws); without it x is updated in every step
+    void* pbuf = nullptr;
+    rc = ensure_ws(h, WS_CGP, og.bytes(h, pp), &pbuf);
+    if (rc && rc != LQ_ERR_NOMEM) return rc;
+    const bool pairs = rc == LQ_OK;
+    const VecRef p2[2] = {v.p, pairs ? og.ref(h, pbuf, pp) : v.p};
     const int Vh = h->g.Vh;
     if (cudaMemsetAsync(e.ptr, 0, og.bytes(h, px), s) != cudaSuccess) return LQ_ERR_CUDA;
     if (pr == px ? cudaMemcpyAsync(v.r.ptr, rhs.ptr, og.bytes(h, px), cudaMemcpyDeviceToDevice, s) != cudaSuccess
@@ -233,7 +237,7 @@ int run_cg(lq_handle* h, const OpGeom& og, const Ctl& c, int pp, const VecRef& e
     if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) rc = LQ_ERR_CUDA;
     for (int k = 0; k < kItersPerGraph && rc == LQ_OK; ++k) {
         // q = K^dag K p, with <p, q> = |K p|^2 and alpha fused into the launch that writes K p
-        const int odd = k & 1;
+        const int odd = pairs ? k & 1 : 0;
         rc = apply_normal(h, og, pp, v.q.ptr, p2[odd].ptr, v.t.ptr, v.tmp.ptr, s, &c);
         if (rc) break;
         if (launch_hop_norm_finalize(c.hop_partial, hop_warps(h, og), og.op == LQ_OP_DWF_NORMAL ? 1 : og.nrhs, c.st,
@@ -242,7 +246,7 @@ int run_cg(lq_handle* h, const OpGeom& og, const Ctl& c, int pp, const VecRef& e
             break;
         }
         if (launch_cg_r_update(v.r, v.q, Vh, og.nblk, og.nrhs, c.sc, c.st, odd, s) != cudaSuccess ||
-            (odd ? launch_cg_x_xpay(e, p2[0], p2[1], v.r, Vh, og.nblk, og.nrhs, c.st, s)
+            (odd || !pairs ? launch_cg_x_xpay(e, p2[0], p2[1], v.r, Vh, og.nblk, og.nrhs, c.st, s)
                  : launch_cg_xpay(p2[1], p2[0], v.r, Vh, og.nblk, og.nrhs, c.st, s)) != cudaSuccess)
             rc = LQ_ERR_CUDA;
     }
