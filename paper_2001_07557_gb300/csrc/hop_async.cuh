@@ -496,8 +496,9 @@ cudaError_t launch_async_threads(const HopArgs& a, cudaStream_t st) {
 // Blocks of 64 threads outside the solvers: twice as many blocks leave the last wave less empty and
 // start as slots of half the size fall free (16^3 x 32 FP32 Schur complement on new inputs each time
 // 19.85 -> 19.35 us, two right-hand sides on the same ones 27.7 -> 26.6; 32^4 FP16 step 139.0 -> 137.7;
-// 16^4 x 16 FP16 domain wall 55.5 -> 53.2).  In the solvers, whose blocks first read their skip flag, 128 are faster (32^4 mixed solve
-// 32.97 against 33.09 ms), and the fused norm's partials are laid out for them.
+// 16^4 x 16 FP16 domain wall 55.5 -> 53.2).  In the solvers, whose blocks first read their skip flag,
+// 128 are faster (32^4 mixed solve 32.97 against 33.09 ms), and the fused norm's partials are laid
+// out for them.
 template <int P, bool R12, bool DAG, int EPI, bool RED>
 cudaError_t launch_async_one(const HopArgs& a, cudaStream_t st) {
     if constexpr (!RED)

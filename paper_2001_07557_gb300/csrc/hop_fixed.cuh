@@ -41,13 +41,13 @@
 // one shared-memory slot each: the next spinor is requested as soon as this one is converted,
 // the next link when this one is used up, so the products (conversions) of a direction cover the
 // latency.  With one thread a site, 168 registers and the 8 directions unrolled, the 120 KB of
-// code kept warps waiting for instructions (240 us); one looped body with run-time directions
-// executed 10,800 instructions a site where this takes 8,900 (236 against 215 us).
+// code kept warps waiting for instructions (240 us against 215); one looped body with run-time
+// directions took 236 us.
 //
 // Measured: D on 32^3 x 16 (as many sites as an even-odd hop of 32^4): 0.92 ms in FP64, 0.214 ms
 // here; its bytes take 0.12 ms.  What bounds it is the integer pipes: without its products,
-// conversions and sums the kernel takes 0.123 ms; the multiplier is busy 64 % of the time, the
-// ALU 44 %, with warps waiting on fixed latencies (ncu).  The sizes cost 1.3 % of a dense field's
+// conversions and sums the kernel takes 0.123 ms; the multiplier is busy 68 % of the time, the
+// ALU 49 %, with warps waiting on fixed latencies (ncu).  The sizes cost 1.3 % of a dense field's
 // time.  Where every site takes slow_site (one spin and colour alone on every site): 0.97 ms; the
 // zero field 0.234, a point source 0.267.
 #pragma once

@@ -11,6 +11,7 @@ import torch
 
 from lqhelp import Handle, dev, host
 from paper_2001_07557_gb300 import inputs, lqcd
+from test_gpu_halo import Slabs
 
 pytestmark = pytest.mark.gpu
 
@@ -41,8 +42,8 @@ def hop(U, psi, dag):
     return -out / 2, size / 2
 
 
-def check(U, psi):
-    with Handle(DIMS, U, mass=-4.0) as H:
+def check(U, psi, U_prec=lqcd.LQ_F64):
+    with Handle(DIMS, U, mass=-4.0, U_prec=U_prec) as H:
         for dag in (False, True):
             x = dev(psi)
             y = torch.empty_like(x)
@@ -101,3 +102,41 @@ def test_sources():
         check(U, psi)
         psi[1:] = 0
         check(U, psi)
+
+
+def test_links_given_in_fp32():
+    for kind in ("random", "near 1"):
+        U = links(kind).astype(np.complex64)
+        psi = 1e-9 * inputs.gaussian_spinor(V, seed=3707)
+        psi[:, 1] *= 1e9
+        check(U, psi, lqcd.LQ_F32)
+
+
+@pytest.mark.parametrize("projected", [False, True])
+def test_slabs_with_ghost_faces(projected):
+    """Sites that take the FP64 sums, and neighbours whose projection is exactly zero, come out of two time
+    slabs bit for bit as out of one lattice."""
+    dims, n = (4, 4, 4, 8), 512
+    U = inputs.gauge_field(dims, "random", seed=3708)
+    g = inputs.gaussian_spinor(n, seed=3709)
+    small, plus, minus, mixed = g.copy(), g.copy(), g.copy(), g * np.exp(-np.arange(n) % 13)[:, None, None]
+    small[:, [0, 2, 3]] *= 1e-8
+    plus[:, 2:] = plus[:, :2]
+    minus[:, 2:] = -minus[:, :2]
+    point, wall = np.zeros_like(g), np.zeros_like(g)
+    point[64 * 4 + 5, 1, 2] = 1
+    wall[256:320, 3, 0] = g[256:320, 3, 0]
+    S = Slabs(dims, 2, U, -4.0, (1, 1, 1, -1), lqcd.LQ_F64)
+    try:
+        with Handle(dims, U, mass=-4.0) as G:
+            for psi in (small, plus, minus, mixed, point, wall):
+                ins = S.scatter(psi)
+                outs = [torch.zeros_like(i) for i in ins]
+                for dag in (False, True):
+                    S.hop(ins, outs, dagger=dag, projected=projected)
+                    x = dev(psi)
+                    y = torch.empty_like(x)
+                    (lqcd.dslash_dag_apply if dag else lqcd.dslash_apply)(G.h, y, x, lqcd.LQ_F64, lqcd.LQ_FULL)
+                    assert np.array_equal(S.gather(outs), host(y))
+    finally:
+        S.close()
