@@ -128,7 +128,7 @@ __device__ __forceinline__ void su3_product(const T2 (&a)[9], const T2 (&b)[9], 
 // on random and smooth links exp(i eps H), eps 0.3 to 1e-6: 4.3 u, as with the FP64 unit alone
 // (a line at 1/64: 6.5 u, at 1/16 4.3 u).
 //
-// 108 FP64 instructions at 77 clocks a warp and SM sub-partition compare with about 1,600 integer and FP32
+// 108 FP64 instructions at 77 clocks a warp and SM sub-partition compare with about 1,800 integer and FP32
 // ones here.  48^4, smooth links: 991 us in FP64, 501 us here (467 where no sum is small, 421 without
 // the sums S; 0.68 of the HBM time of its bytes), with three blocks an SM and in place.  Where all of every pair
 // goes to the FP64 unit: 1027-1045 us; A = 1 and a smooth B 1049.  S after the fixed-point product: 483 and
