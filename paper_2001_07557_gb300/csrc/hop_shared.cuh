@@ -286,13 +286,19 @@ __global__ void __launch_bounds__(kShSites* G, shared_min_blocks<P, G>()) wilson
             }
         }
         if constexpr (EPI == EPI_DWF) {
-            const HopShift<T> sh = hop_shift<DAG, T>(a, rhs);
+            const int Ls = a.Ls, sl = rhs;
+            const int s_up = DAG ? (sl + 1 == Ls ? 0 : sl + 1) : (sl == 0 ? Ls - 1 : sl - 1);
+            const int s_dn = DAG ? (sl == 0 ? Ls - 1 : sl - 1) : (sl + 1 == Ls ? 0 : sl + 1);
+            const bool wrap_up = DAG ? (sl + 1 == Ls) : (sl == 0);
+            const bool wrap_dn = DAG ? (sl == 0) : (sl + 1 == Ls);
+            const T c_up = wrap_up ? (T)(-a.c_shift * a.mf) : (T)a.c_shift;
+            const T c_dn = wrap_dn ? (T)(-a.c_shift * a.mf) : (T)a.c_shift;
             cplx<T> su[6], sd[6];
             T nu, nd;
-            // only P+ psi(sh.up) (spins 0,1) and P- psi(sh.dn) (spins 2,3) are needed
-            load_half_spinor_raw<P, true>(a.x[p] + (size_t)sh.up * a.x_rhs, g.Vh, i, su, nu);
-            load_half_spinor_raw<P, false>(a.x[p] + (size_t)sh.dn * a.x_rhs, g.Vh, i, sd, nd);
-            const T cu = sh.c_up * nu, cdn = sh.c_dn * nd;
+            // only P+ psi(s_up) (spins 0,1) and P- psi(s_dn) (spins 2,3) are needed
+            load_half_spinor_raw<P, true>(a.x[p] + (size_t)s_up * a.x_rhs, g.Vh, i, su, nu);
+            load_half_spinor_raw<P, false>(a.x[p] + (size_t)s_dn * a.x_rhs, g.Vh, i, sd, nd);
+            const T cu = c_up * nu, cdn = c_dn * nd;
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
                 o[k].re = fma(cu, su[k].re, o[k].re);

@@ -53,8 +53,9 @@ struct HopArgs {
 
 // c_shift (S x)(s): P+ = upper spins (gamma_5 = diag(1,1,-1,-1)).  Non-dagger: upper from
 // s-1, lower from s+1; dagger swaps.  Coefficient c_shift (Shamir: -1), times -mf across the wall.
-// (hop_async.cuh and hop_mma.cuh spell it out, which compiles better there: 16^4 x 16 FP16 53.2 and
-// 164 us against 54.2 and 166; hop_shared.cuh, FP32, D^dag: 71.6 us spelt out, 70.0 with this.)
+// hop_async.cuh, hop_shared.cuh and hop_mma.cuh spell it out, which compiles better there: 16^4 x 16 FP16
+// 53.2 us and, on the tensor cores, 164 against 54.2 and 166 with this; FP32 even-odd Moebius operator on
+// 18 x 16 x 18 x 10 x 16 133.9 against 135.3 (D^dag on 16^4 x 16 alone gained, 71.6 -> 70.0).
 template <typename T>
 struct HopShift {
     int up, dn;     // slices that the upper and the lower spins come from
